@@ -5,9 +5,18 @@
 // Real embedding: with Y_f = [Re Qhat_f ; Im Qhat_f] (2nb rows x points, K-major
 // in HBM; sqrt(W) is already folded into Qhat), D = Y_f Y_f^T gives
 //   Re M_f[l][l'] = D[l][l'] + D[nb+l][nb+l'],  Im M_f[l][l'] = D[l][nb+l'] - D[nb+l][l'].
-// An item is two 64-point blocks of one frequency; its stage holds the TMA
-// boxes (NP rows x 64 points x 2 blocks, NP = 2nb rounded up to 16, 128-byte
-// swizzle) of hi and, for BF16X3, of lo.  Per K step of 16 (N = NP):
+// An item is kpb 64-point blocks of one frequency; its stage holds the TMA
+// boxes (NP rows x 64 points x kpb blocks, NP = 2nb rounded up to 16, 128-byte
+// swizzle) of hi and, for BF16X3, of lo.  The MMA always has M = 128 rows, so
+// with NP <= 64 it takes P = 128 / NP consecutive blocks of the stage at once
+// (their rows are contiguous): A = B = the P x NP stacked rows, N = P x NP, and
+// of D only the P diagonal NP x NP blocks are read, one A1 run per block each
+// as before (the same MMAs on the same rows, so the same rounding).  A stage,
+// an MMA group and a drain then cover P blocks: with 16 rows (nb = 7) a
+// 64-point block is 4 KB, and one hand-over per block left the kernel waiting
+// for its hand-overs: 361 x 720 x 2 points, 361 bins, nb = 7, bf16x3 took
+// 11.5 ms and takes 2.3 (4.8 TB/s of Qhat); with 48 rows (nb = 21, 193 bins)
+// 6.2 -> 3.5 ms.  Per K step of 16:
 //   A1 (+)= hi hi^T   restarted every `flush` blocks (short FP32 runs in the
 //                      tensor core), drained into Kahan-compensated registers.
 //                      The tensor core's FP32 accumulation rounds toward zero,
@@ -44,7 +53,12 @@ namespace spod {
 namespace {
 
 constexpr int kMaxStages = 8;
-constexpr int kKpb = 2;                   // 64-point blocks per item (one TMA copy per operand)
+// 64-point blocks per MMA (stacked diagonal blocks of D) for np rows per block
+__host__ __device__ constexpr int gram_pack(int np) { return np <= 64 ? 128 / np : 1; }
+// 64-point blocks per item (one TMA copy per operand): whole MMA packs, and at
+// least two blocks (with 80 rows, items of one block measured 6.88 ms against
+// 6.79 on the 512 x 256 x 3 grid)
+__host__ __device__ constexpr int gram_kpb(int np) { return gram_pack(np) > 2 ? gram_pack(np) : 2; }
 constexpr int kEpiWarps = 8;
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1, kDiagWarp0 = kEpiWarps + 2;
@@ -55,10 +69,10 @@ constexpr int kMaxAcc = 4;                // A1 accumulator buffers at most
 
 struct GramTcArgs {
   int nb, r2, np, nf;
-  int64_t nkb;                            // items (block pairs) per frequency in this chunk
-  int64_t nblk;                           // 64-point blocks per frequency in this chunk
+  int64_t nkb;                            // items per frequency in this chunk
+  int64_t nsb;                            // packs of P 64-point blocks per frequency in this chunk
   int64_t nitems;                         // nf * nkb
-  int flush;                              // 64-point blocks per A1 run
+  int flush;                              // packs (64-point blocks of one diagonal block) per A1 run
   int nacc;                               // A1 buffers in tensor memory (2..kMaxAcc, as np allows)
   int stall0;                             // self-test: the first item's copies are never issued, so
                                           // every wait on them runs out (the bounded-wait path)
@@ -110,10 +124,10 @@ struct GramHdr {
   int abort;
 };
 
-// Walks the group and segment structure of a CTA's range, one 64-point
-// block at a time: a segment is the run of one frequency, a group (one A1
-// run in tensor memory) at most `flush` consecutive blocks of a segment; a
-// group may end inside an item.  All roles step it identically.
+// Walks the group and segment structure of a CTA's range, one pack (P
+// 64-point blocks) at a time: a segment is the run of one frequency, a group
+// (one A1 run in tensor memory) at most `flush` consecutive packs of a
+// segment; a group may end inside an item.  All roles step it identically.
 struct GroupWalk {
   int fprev = -1;
   int in_group = 0;
@@ -154,9 +168,13 @@ struct Cursor {
   }
 };
 
-// Slot layout (bytes): A1 (sum, carry) pairs [r2][r2] float2, A2 [r2][r2]
-// float, then the lo-square diagonal [r2] float.
-__host__ __device__ inline size_t gram_slot_bytes(int r2) { return (size_t)r2 * r2 * 12 + (size_t)r2 * 4; }
+// Slot of one (CTA, frequency): P sub-slots, one per diagonal block of D.
+// Sub-slot layout (bytes): A1 (sum, carry) pairs [r2][r2] float2, A2 [r2][r2]
+// float, then (sub-slot 0 only) the lo-square diagonal [r2] float; whole
+// 8-byte words, so that every sub-slot's pairs are aligned.
+__host__ __device__ inline size_t gram_slot_bytes(int r2) {
+  return ((size_t)r2 * r2 * 12 + (size_t)r2 * 4 + 7) / 8 * 8;
+}
 
 template <bool X3, int HC>
 __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_constant__ CUtensorMap map_hi,
@@ -164,11 +182,12 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
                                                    uint8_t* __restrict__ slots, unsigned* __restrict__ gflags) {
   using namespace tc;
   constexpr int NOPS = X3 ? 2 : 1;
+  constexpr int NP = 2 * HC, P = gram_pack(NP), KPB = gram_kpb(NP), KSB = KPB / P;
   extern __shared__ unsigned char smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   GramHdr* hdr = reinterpret_cast<GramHdr*>(sm);
   uint8_t* stages = sm + 1024;
-  const uint32_t op_bytes = a.box_bytes * kKpb;          // one operand of an item
+  const uint32_t op_bytes = a.box_bytes * KPB;           // one operand of an item
   const uint32_t stage_bytes = op_bytes * NOPS;          // [hi blocks][lo blocks]
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -176,7 +195,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
   const int64_t i1 = a.nitems * (blockIdx.x + 1) / gridDim.x;
   const int nit = (int)(i1 - i0);
   const int FB = a.flush;
-  const int nkb = (int)a.nkb, nblk = (int)a.nblk;
+  const int nkb = (int)a.nkb, nsb = (int)a.nsb;
 
   if (tid == 0) {
     for (int i = 0; i < a.nst; ++i) {
@@ -223,8 +242,8 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       const uint32_t fb = smem_u32(&hdr->full[s]);
       mbar_arrive_expect_tx(fb, stage_bytes);
       uint8_t* st = stages + (size_t)s * stage_bytes;
-      tma_load_4d(smem_u32(st), &map_hi, 0, 0, cu.f, cu.kp * kKpb, fb);
-      if (X3) tma_load_4d(smem_u32(st + op_bytes), &map_lo, 0, 0, cu.f, cu.kp * kKpb, fb);
+      tma_load_4d(smem_u32(st), &map_hi, 0, 0, cu.f, cu.kp * KPB, fb);
+      if (X3) tma_load_4d(smem_u32(st + op_bytes), &map_lo, 0, 0, cu.f, cu.kp * KPB, fb);
       issued = i + 1;
     }
     // copies still in flight must land before the CTA can exit
@@ -232,7 +251,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       mbar_drain(smem_u32(&hdr->full[i % a.nst]), (i / a.nst) & 1, gflags);
   } else if (warp == kMmaWarp && lane == 0 && nit > 0) {
     // ---------------- MMA issuer
-    const uint32_t idesc = idesc_bf16(128, a.np, 0, 0);
+    const uint32_t idesc = idesc_bf16(128, P * NP, 0, 0);
     GroupWalk gw;
     Cursor cu;
     cu.init(i0, nkb);
@@ -243,8 +262,9 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       if (!mbar_wait(smem_u32(&hdr->full[s]), cu.ph, abort_flag, gflags)) break;
       tc_fence_after();
       const uint32_t st = smem_u32(stages + (size_t)s * stage_bytes);
-      // a block past the chunk's points (odd block count) holds no data of this chunk
-      const int nvalid = min(kKpb, nblk - kp * kKpb);
+      // packs past the chunk's last one hold no data (blocks past the chunk's
+      // last one read as zeros)
+      const int nvalid = min(KSB, nsb - kp * KSB);
       const bool item_last = i + 1 == nit || cu.last_of_f(nkb);
       for (int j = 0; j < nvalid; ++j) {
         const bool gstart = gw.step(f, FB, a.nacc);
@@ -263,9 +283,9 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
           break;
         }
         tc_fence_after();
-        const uint32_t d1 = tmem + (uint32_t)(acc * a.np);
-        const uint32_t d2 = tmem + (uint32_t)((a.nacc + a2b) * a.np);
-        const uint32_t hi = st + (uint32_t)j * a.box_bytes;
+        const uint32_t d1 = tmem + (uint32_t)(acc * P * NP);
+        const uint32_t d2 = tmem + (uint32_t)((a.nacc + a2b) * P * NP);
+        const uint32_t hi = st + (uint32_t)(j * P) * a.box_bytes;
         const uint32_t lo = hi + op_bytes;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -291,7 +311,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
     // shuffles when the CTA's run of a frequency ends.
     const int t = tid - kDiagWarp0 * 32;
     const int rsub = t >> 3, chunk = t & 7;
-    constexpr int kRowsPer = 16;                      // rows rsub + 8 j, j < 16: up to 128 rows
+    constexpr int kRowsPer = NP / 8;                  // rows rsub + 8 j < NP
     float q[kRowsPer];
 #pragma unroll
     for (int j = 0; j < kRowsPer; ++j) q[j] = 0.f;
@@ -302,7 +322,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       const bool send = i + 1 == nit || cu.last_of_f(nkb);
       const int s = cu.s;
       if (!mbar_wait(smem_u32(&hdr->full[s]), cu.ph, abort_flag, gflags)) break;
-      const int nvalid = min(kKpb, nblk - kp * kKpb);
+      const int nvalid = min(KSB, nsb - kp * KSB) * P;
       for (int b = 0; b < nvalid; ++b) {
         const uint8_t* lo = stages + (size_t)s * stage_bytes + op_bytes + (size_t)b * a.box_bytes;
 #pragma unroll
@@ -324,7 +344,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       }
       mbar_arrive(smem_u32(&hdr->empty[s]));
       if (send) {
-        float* dg = reinterpret_cast<float*>(slots + ((size_t)blockIdx.x + (size_t)f) * gram_slot_bytes(a.r2) +
+        float* dg = reinterpret_cast<float*>(slots + ((size_t)blockIdx.x + (size_t)f) * P * gram_slot_bytes(a.r2) +
                                              (size_t)a.r2 * a.r2 * 12);
 #pragma unroll
         for (int j = 0; j < kRowsPer; ++j) {
@@ -339,18 +359,27 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       }
     }
   } else if (warp < kEpiWarps) {
-    // ---------------- epilogue: TMEM -> registers -> slots.  Warp (quad,
-    // half) drains rows quad*32 .. +31 and the HC columns of its half; of A1
-    // (symmetric) only the 8-column chunks that reach the upper triangle
-    // (some row of the quad <= some column of the chunk) are read and summed.
+    // ---------------- epilogue: TMEM -> registers -> slots.  Lane (quad, lane)
+    // holds row 32 quad + lane of D: row lr of diagonal block sub.  Warp (quad,
+    // half) drains the HC columns of its half of that block; where the quad
+    // spans two diagonal blocks (they change at lane 16: NP is a multiple of
+    // 16) both blocks' columns are read and each lane keeps its own.  Of A1
+    // (symmetric) only the 8-column chunks that reach the upper triangle (some
+    // row of the warp <= some column of the chunk) are read and summed.
     constexpr int CH = HC / 8;
+    constexpr bool kTwo = P > 1 && NP % 32 != 0;  // some quad spans two diagonal blocks
     const int quad = warp & 3, half = warp >> 2;
-    const int row = quad * 32 + lane;
+    const int sub_lo = quad * 32 / NP, sub_hi = (quad * 32 + 16) / NP;
+    const bool two = kTwo && sub_hi != sub_lo && sub_hi < P;
+    const bool upper = two && lane >= 16;
+    const int sub = upper ? sub_hi : sub_lo;
+    const int row = quad * 32 + lane - sub * NP;  // row of the lane's diagonal block
+    const int rmin = two ? 0 : quad * 32 - sub_lo * NP;
     const int col0 = half * HC;
-    const bool active = quad * 32 < a.r2;         // this lane quadrant holds rows of D
+    const bool active = sub_lo < P && (two || rmin < a.r2);   // this lane quadrant holds rows of D
     int nch = 0;                                  // chunks [CH - nch, CH) of this warp are upper-triangle ones
 #pragma unroll
-    for (int c = 0; c < CH; ++c) nch += (col0 + 8 * c + 7 >= quad * 32) ? 1 : 0;
+    for (int c = 0; c < CH; ++c) nch += (col0 + 8 * c + 7 >= rmin) ? 1 : 0;
     const int c_first = CH - nch;
     float s1[HC], c1[HC];
 #pragma unroll
@@ -361,7 +390,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
     bool ok = true;
     for (int i = 0; i < nit && ok; ++i, cu.next(nkb, a.nst)) {
      const int f = cu.f;
-     const int nvalid = min(kKpb, nblk - cu.kp * kKpb);
+     const int nvalid = min(KSB, nsb - cu.kp * KSB);
      const bool item_last = i + 1 == nit || cu.last_of_f(nkb);
      for (int j = 0; j < nvalid; ++j) {
       gw.step(f, FB, a.nacc);
@@ -378,12 +407,23 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       tc_fence_after();
       if (active && nch > 0) {
         // this warp's A1 chunks in one batch of loads and one wait
-        const uint32_t t1 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * a.np) + (uint32_t)col0;
+        const uint32_t t1 =
+            tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * P * NP + sub_lo * NP) + (uint32_t)col0;
         float v[HC];
 #pragma unroll
         for (int c = 0; c < CH; ++c)
           if (c >= c_first) tmem_ld8(t1 + (uint32_t)(c * 8), v + c * 8);
-        tmem_wait_ld();
+        if (kTwo && two) {
+          float w[HC];
+#pragma unroll
+          for (int c = 0; c < CH; ++c)
+            if (c >= c_first) tmem_ld8(t1 + (uint32_t)(NP + c * 8), w + c * 8);
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < HC; ++c) v[c] = upper ? w[c] : v[c];
+        } else {
+          tmem_wait_ld();
+        }
         tc_fence_before();
         mbar_arrive(smem_u32(&hdr->accempty[acc]));
 #pragma unroll
@@ -400,8 +440,8 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       }
       if (!send) continue;
       // the CTA's run of frequency f ends: its sums go to slot (cta + f)
-      uint8_t* slot = slots + ((size_t)blockIdx.x + (size_t)f) * gram_slot_bytes(a.r2);
-      const bool wr = row < a.r2;
+      uint8_t* slot = slots + (((size_t)blockIdx.x + (size_t)f) * P + sub) * gram_slot_bytes(a.r2);
+      const bool wr = row < a.r2 && sub < P;
       if (active) {
         float2* d1 = reinterpret_cast<float2*>(slot) + (size_t)row * a.r2 + col0;
 #pragma unroll
@@ -414,12 +454,21 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       if (X3) {
         if (active) {
           // the segment's A2 (its MMAs completed with the last group's), not symmetric: all of it
-          const uint32_t t2 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((a.nacc + a2b) * a.np) +
-                              (uint32_t)col0;
+          const uint32_t t2 = tmem + ((uint32_t)(quad * 32) << 16) +
+                              (uint32_t)((a.nacc + a2b) * P * NP + sub_lo * NP) + (uint32_t)col0;
           float v[HC];
 #pragma unroll
           for (int c = 0; c < CH; ++c) tmem_ld8(t2 + (uint32_t)(c * 8), v + c * 8);
-          tmem_wait_ld();
+          if (kTwo && two) {
+            float w[HC];
+#pragma unroll
+            for (int c = 0; c < CH; ++c) tmem_ld8(t2 + (uint32_t)(NP + c * 8), w + c * 8);
+            tmem_wait_ld();
+#pragma unroll
+            for (int c = 0; c < HC; ++c) v[c] = upper ? w[c] : v[c];
+          } else {
+            tmem_wait_ld();
+          }
           tc_fence_before();
           mbar_arrive(smem_u32(&hdr->a2empty[a2b]));
           float* d2 = reinterpret_cast<float*>(slot + (size_t)a.r2 * a.r2 * 8) + (size_t)row * a.r2 + col0;
@@ -445,32 +494,45 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
 // CTA c's item range is [floor(c W / G), floor((c+1) W / G)); the CTA holding item i.
 __device__ __forceinline__ int64_t cta_of_item(int64_t i, int64_t W, int64_t G) { return ((i + 1) * G - 1) / W; }
 
-// acc[f] (+)= sum over the CTAs c that covered frequency f of slot (c + f), in
-// CTA order, of D = A1 + A2 + A2^T + diag(lo lo^T) (A1 as a compensated (sum, carry)
-// pair, read from its upper triangle).
-__global__ void k_gram_tc_collect(const uint8_t* __restrict__ slots, int r2, int64_t nkb, int64_t G, int x3,
-                                  int first, double* __restrict__ acc) {
+// acc[f] (+)= sum over the CTAs c that covered frequency f of the pack
+// sub-slots of slot (c + f), in CTA and sub-slot order, of D = A1 + A2 + A2^T +
+// diag(lo lo^T) (A1 as a compensated (sum, carry) pair, read from its upper triangle).
+__global__ void k_gram_tc_collect(const uint8_t* __restrict__ slots, int r2, int pack, int64_t nkb, int64_t G,
+                                  int x3, int first, double* __restrict__ acc) {
   const int f = blockIdx.x;
   const int64_t W = (int64_t)gridDim.x * nkb;
   const int64_t c0 = cta_of_item((int64_t)f * nkb, W, G);
   const int64_t c1 = cta_of_item((int64_t)(f + 1) * nkb - 1, W, G);
   double* dst = acc + (int64_t)f * r2 * r2;
   const size_t sb = gram_slot_bytes(r2);
-  for (int e = threadIdx.x; e < r2 * r2; e += blockDim.x) {
-    const int i = e / r2, j = e - i * r2;
+  // one entry (i <= j) of the symmetric D per thread: the conversions and sums
+  // in FP64 bound this kernel
+  const int t = blockIdx.y * blockDim.x + threadIdx.x;
+  if (t < r2 * (r2 + 1) / 2) {
+    int j = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    while (j * (j + 1) / 2 > t) --j;
+    while ((j + 1) * (j + 2) / 2 <= t) ++j;
+    const int i = t - j * (j + 1) / 2;
+    const int e = i * r2 + j;
     double v = 0.0;
-    for (int64_t c = c0; c <= c1; ++c) {
-      const uint8_t* slot = slots + (size_t)(c + f) * sb;
-      // A1 is symmetric and only its upper triangle is summed by the epilogue
-      const float2 sc = reinterpret_cast<const float2*>(slot)[i <= j ? e : j * r2 + i];
-      v += (double)sc.x + (double)sc.y;
-      if (x3) {
-        const float* a2 = reinterpret_cast<const float*>(slot + (size_t)r2 * r2 * 8);
-        v += (double)a2[e] + (double)a2[j * r2 + i];
-        if (i == j) v += (double)reinterpret_cast<const float*>(slot + (size_t)r2 * r2 * 12)[i];
+    const int et = j * r2 + i;
+    const size_t o2 = (size_t)r2 * r2 * 8;
+    const uint8_t* slot = slots + (size_t)(c0 + f) * pack * sb;
+    for (int c = 0; c <= (int)(c1 - c0); ++c) {
+      if (x3 && i == j) v += (double)reinterpret_cast<const float*>(slot + o2 + (size_t)r2 * r2 * 4)[i];
+#pragma unroll 8
+      for (int q = 0; q < pack; ++q, slot += sb) {
+        const float2 sc = reinterpret_cast<const float2*>(slot)[e];   // A1: upper triangle only
+        v += (double)sc.x + (double)sc.y;
+        if (x3) {
+          const float* a2 = reinterpret_cast<const float*>(slot + o2);
+          v += (double)a2[e] + (double)a2[et];
+        }
       }
     }
-    dst[e] = first ? v : dst[e] + v;
+    v = first ? v : dst[e] + v;
+    dst[e] = v;
+    dst[et] = v;
   }
 }
 
@@ -495,7 +557,8 @@ __global__ void k_gram_tc_finish(const double* __restrict__ acc, int nb, int r2,
     }
     return v;
   };
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
+  const int e = blockIdx.y * blockDim.x + threadIdx.x;   // one entry per thread
+  if (e < nb * nb) {
     const int i = e / nb, j = e - i * nb;
     const int l = min(i, j), lp = max(i, j);
     double vr = dc(l, lp) + dc(nb + l, nb + lp);
@@ -517,30 +580,32 @@ size_t gram_tc_smem_stages(const spod_plan_s& p, int nst) {
   const int nops = p.desc.precision == SPOD_PREC_BF16X3 ? 2 : 1;
   const size_t np = (size_t)((2 * p.nb + 15) / 16 * 16);
   // + the rows an M = 128 A operand reads past the last stage's last block
-  return 1024 + 1024 + (size_t)nst * nops * kKpb * np * 128 + (128 - np) * 128;
+  return 1024 + 1024 + (size_t)nst * nops * gram_kpb((int)np) * np * 128 + (128 - gram_pack((int)np) * np) * 128;
 }
 
 template <bool X3, int HC>
-cudaError_t launch_gram_tc_t(const spod_plan_s& p, const GramTcArgs& a, int grid, size_t smem, cudaStream_t s) {
+cudaError_t launch_gram_tc_t(const spod_plan_s& p, const CUtensorMap& map_hi, const CUtensorMap& map_lo,
+                             const GramTcArgs& a, int grid, size_t smem, cudaStream_t s) {
   auto kern = k_gram_tc<X3, HC>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kThreadsGram, smem, s>>>(p.tmap_hi2, X3 ? p.tmap_lo2 : p.tmap_hi2, a,
+  kern<<<grid, kThreadsGram, smem, s>>>(map_hi, X3 ? map_lo : map_hi, a,
                                         reinterpret_cast<uint8_t*>(p.d_gslot), p.d_flags);
   return cudaGetLastError();
 }
 
 template <bool X3>
-cudaError_t launch_gram_tc_x(const spod_plan_s& p, const GramTcArgs& a, int grid, size_t smem, cudaStream_t s) {
+cudaError_t launch_gram_tc_x(const spod_plan_s& p, const CUtensorMap& mh, const CUtensorMap& ml, const GramTcArgs& a,
+                             int grid, size_t smem, cudaStream_t s) {
   switch (a.np / 2) {                      // columns per epilogue warp (np is a multiple of 16)
-    case 8: return launch_gram_tc_t<X3, 8>(p, a, grid, smem, s);
-    case 16: return launch_gram_tc_t<X3, 16>(p, a, grid, smem, s);
-    case 24: return launch_gram_tc_t<X3, 24>(p, a, grid, smem, s);
-    case 32: return launch_gram_tc_t<X3, 32>(p, a, grid, smem, s);
-    case 40: return launch_gram_tc_t<X3, 40>(p, a, grid, smem, s);
-    case 48: return launch_gram_tc_t<X3, 48>(p, a, grid, smem, s);
-    case 56: return launch_gram_tc_t<X3, 56>(p, a, grid, smem, s);
-    case 64: return launch_gram_tc_t<X3, 64>(p, a, grid, smem, s);
+    case 8: return launch_gram_tc_t<X3, 8>(p, mh, ml, a, grid, smem, s);
+    case 16: return launch_gram_tc_t<X3, 16>(p, mh, ml, a, grid, smem, s);
+    case 24: return launch_gram_tc_t<X3, 24>(p, mh, ml, a, grid, smem, s);
+    case 32: return launch_gram_tc_t<X3, 32>(p, mh, ml, a, grid, smem, s);
+    case 40: return launch_gram_tc_t<X3, 40>(p, mh, ml, a, grid, smem, s);
+    case 48: return launch_gram_tc_t<X3, 48>(p, mh, ml, a, grid, smem, s);
+    case 56: return launch_gram_tc_t<X3, 56>(p, mh, ml, a, grid, smem, s);
+    case 64: return launch_gram_tc_t<X3, 64>(p, mh, ml, a, grid, smem, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -550,11 +615,11 @@ cudaError_t launch_gram_tc_x(const spod_plan_s& p, const GramTcArgs& a, int grid
 // Shared memory of the smallest (2-stage) configuration; launches use up to 8 stages.
 size_t gram_tc_smem_bytes(const spod_plan_s& p) { return gram_tc_smem_stages(p, 2); }
 
-// Slots of the persistent kernel, (max CTAs + nf - 1) x gram_slot_bytes(qrows)
+// Slots of the persistent kernel, (max CTAs + nf - 1) x pack x gram_slot_bytes(qrows)
 // (counted in doubles), and the per-frequency FP64 accumulator of D over
 // chunks, nf x qrows^2 (qrows = 2 nb, + 1 with the folded mean's rho row).
 size_t gram_tc_slot_doubles(const spod_plan_s& p, int max_ctas) {
-  return ((size_t)(max_ctas + p.nf - 1) * gram_slot_bytes(p.qrows) + 7) / 8;
+  return (size_t)(max_ctas + p.nf - 1) * gram_pack((2 * p.nb + 15) / 16 * 16) * gram_slot_bytes(p.qrows) / 8;
 }
 size_t gram_tc_acc_doubles(const spod_plan_s& p) { return (size_t)p.nf * p.qrows * p.qrows; }
 
@@ -573,12 +638,14 @@ cudaError_t launch_gram_tc_chunk(const spod_plan_s& p, int64_t mcount, bool firs
   a.flush = p.gram_flush > 0 ? p.gram_flush : 1;
   a.box_bytes = (uint32_t)a.np * 128u;
   // A1 buffers: as many as the 512 tensor-memory columns hold beside the two
-  // A2 buffers (np = 80 for nb = 38: four), so that short A1 runs are drained
-  // while the next ones accumulate
-  a.nacc = std::max(2, std::min(kMaxAcc, ((int)kTmemCols - 2 * a.np) / a.np));
+  // A2 buffers (np = 80 for nb = 38: four; packed blocks: two or three of P
+  // blocks each), so that short A1 runs are drained while the next ones accumulate
+  const int pack = gram_pack(a.np), kpb = gram_kpb(a.np), ncol = pack * a.np;
+  a.nacc = std::max(2, std::min(kMaxAcc, ((int)kTmemCols - 2 * ncol) / ncol));
   a.stall0 = p.wait_selftest ? 1 : 0;
-  a.nblk = (mcount + 63) / 64;
-  a.nkb = (a.nblk + kKpb - 1) / kKpb;
+  const int64_t nblk = (mcount + 63) / 64;
+  a.nsb = (nblk + pack - 1) / pack;
+  a.nkb = (nblk + kpb - 1) / kpb;
   a.nitems = a.nkb * p.nf;
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p.device);
@@ -586,16 +653,22 @@ cudaError_t launch_gram_tc_chunk(const spod_plan_s& p, int64_t mcount, bool firs
   while (a.nst > 2 && gram_tc_smem_stages(p, a.nst) > (size_t)optin) --a.nst;
   const size_t smem = gram_tc_smem_stages(p, a.nst);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(gram_tc_ctas(p), a.nitems));
-  cudaError_t e = p.desc.precision == SPOD_PREC_BF16X3 ? launch_gram_tc_x<true>(p, a, grid, smem, s)
-                                                        : launch_gram_tc_x<false>(p, a, grid, smem, s);
+  // maps whose last block is the chunk's: what a box reads past it is zero
+  CUtensorMap mh, ml;
+  if (!make_qhat_map(p, p.d_qhat, kpb, nblk, &mh) || !make_qhat_map(p, p.d_qlo ? p.d_qlo : p.d_qhat, kpb, nblk, &ml))
+    return cudaErrorUnknown;
+  cudaError_t e = p.desc.precision == SPOD_PREC_BF16X3 ? launch_gram_tc_x<true>(p, mh, ml, a, grid, smem, s)
+                                                        : launch_gram_tc_x<false>(p, mh, ml, a, grid, smem, s);
   if (e != cudaSuccess) return e;
-  k_gram_tc_collect<<<p.nf, 256, 0, s>>>(reinterpret_cast<const uint8_t*>(p.d_gslot), a.r2, a.nkb, grid,
+  k_gram_tc_collect<<<dim3((unsigned)p.nf, (unsigned)((a.r2 * (a.r2 + 1) / 2 + 127) / 128)), 128, 0, s>>>(
+      reinterpret_cast<const uint8_t*>(p.d_gslot), a.r2, pack, a.nkb, grid,
                                          p.desc.precision == SPOD_PREC_BF16X3 ? 1 : 0, first ? 1 : 0, p.d_gacc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gram_tc_finish(const spod_plan_s& p, cudaStream_t s) {
-  k_gram_tc_finish<<<p.nf, 256, 0, s>>>(p.d_gacc, p.nb, p.qrows, p.mean_fold ? p.d_what : nullptr, p.kappa,
+  k_gram_tc_finish<<<dim3((unsigned)p.nf, (unsigned)((p.nb * p.nb + 255) / 256)), 256, 0, s>>>(
+      p.d_gacc, p.nb, p.qrows, p.mean_fold ? p.d_what : nullptr, p.kappa,
                                         p.d_gram, p.d_flags);
   return cudaGetLastError();
 }

@@ -18,10 +18,17 @@
 // adjoint.
 //
 // Persistent CTAs (one per SM) walk a contiguous range of the f-major list of
-// (frequency, 128-point tile) items.  Warp roles (320 threads): warp 8 issues
-// TMA (and the B image copy at each frequency change), warp 9 issues the MMAs
-// into two TMEM accumulators, warps 0-7 drain them (warps w and w+4 share a
-// lane quadrant and take one half of the columns each).  Every wait is bounded.
+// (frequency, group of 128-point tiles) items.  Warp roles (576 threads): warp 16
+// issues TMA (and the B image copy at each frequency change), warp 17 issues the
+// MMAs into four TMEM accumulators, four groups of four warps (one warp per
+// lane quadrant) drain the items in turn.  Every wait is bounded.
+//
+// What bounds it: HBM (Qhat read, Phi written), as long as enough bytes are in
+// flight and no tile waits for a hand-over.  Hence items of about 32 KB whatever
+// nb is, one hand-over per item, and sixteen draining warps: 361 x 720 x 2
+// points, 361 bins, nb = 7, three modes 10.7 -> 2.6 ms (6.0 TB/s); nb = 21, 193
+// bins, five modes 6.1 -> 3.6 ms; 512 x 256 x 3 points, nb = 38, five modes
+// 6.5 -> 5.2 ms (6.7 TB/s), 38 modes of a quarter of it 2.62 -> 2.46 ms.
 #include <algorithm>
 
 #include "tc_common.cuh"
@@ -29,11 +36,15 @@
 namespace spod {
 namespace {
 
-constexpr int kMaxStages = 4;            // pipeline depth (fewer when shared memory is short)
+constexpr int kMaxStages = 8;            // pipeline depth (fewer when shared memory is short)
+constexpr int kStageTarget = 32 * 1024;  // bytes of an item's stage: as many 128-point tiles as fit (at least one)
+constexpr int kMaxTiles = 8;             // 128-point tiles per item at most
 constexpr int kMaxImageModes = 128;      // modes of one image (nmodes <= nb; the tensor path keeps 2 nb <= 128)
-constexpr uint32_t kTmemCols = 256;       // two accumulators at columns 0 and 128
-constexpr int kEpiWarps = 8;
-constexpr int kEpiThreads = kEpiWarps * 32;
+constexpr int kAcc = 4;                   // TMEM accumulators, 128 columns apart (all tiles of an item)
+constexpr uint32_t kTmemCols = kAcc * 128;
+constexpr int kEpiWarps = 16;
+constexpr int kEpiGroups = kEpiWarps / 4;
+constexpr int kEpiThreads = 4 * 32;                // one group of four warps drains an item
 constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
 constexpr int kThreadsModes = (kEpiWarps + 2) * 32;
 
@@ -42,8 +53,10 @@ struct ModesTcArgs {
   int64_t mcount, m0, M;                  // M: row stride of Phi in points
   int64_t phioff;                          // point of Phi's first column (tiled output)
   int64_t ntp;                             // 128-point tiles per frequency
+  int64_t nit;                             // items (of `tiles` tiles) per frequency
+  int tiles;                               // 128-point tiles per item
   int64_t qtile0;                          // first 128-point tile of the call inside the Qhat chunk
-  int64_t nitems;                          // (f1 - f0) * ntp
+  int64_t nitems;                          // (f1 - f0) * nit
   int f0;                                  // first frequency of the call's range
   uint32_t box_bytes;                      // one Qhat TMA box: np rows x 128 bytes
   uint32_t img_bytes;                      // one B image (hi or lo)
@@ -51,7 +64,7 @@ struct ModesTcArgs {
 };
 
 struct ModesHdr {
-  uint64_t full[kMaxStages], empty[kMaxStages], accfull[2], accempty[2], bfull, bempty, drain;
+  uint64_t full[kMaxStages], empty[kMaxStages], accfull[kAcc], accempty[kAcc], bfull, bempty, drain;
   uint32_t tmem_base;
   int abort;
 };
@@ -130,7 +143,7 @@ __global__ void k_mode_image(const float* __restrict__ bmat, int nb, int nm, int
 // ring, advanced without divisions (the issuing threads are on the critical
 // path of every item).
 struct Cursor {
-  int f, tp;          // frequency, 128-point tile within it
+  int f, tp;          // frequency, item (group of tiles) within it
   int s, ph;          // stage, parity of the ring pass (i / nst) & 1
   __device__ __forceinline__ void init(int64_t item0, int ntp, int f0) {
     const int fr = (int)(item0 / ntp);
@@ -157,21 +170,23 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
   ModesHdr* hdr = reinterpret_cast<ModesHdr*>(sm);
   uint8_t* Bhi = sm + 1024;
   uint8_t* Blo = Bhi + a.img_bytes;
-  const uint32_t stage_bytes = 2u * a.box_bytes * NOPS;   // two 64-point boxes (hi [, lo])
+  const uint32_t tile_bytes = 2u * a.box_bytes;           // a tile's two 64-point boxes of one operand
+  const uint32_t op_bytes = tile_bytes * a.tiles;
+  const uint32_t stage_bytes = op_bytes * NOPS;           // [hi tiles][lo tiles]
   uint8_t* stages = Bhi + NOPS * a.img_bytes;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t i0 = a.nitems * blockIdx.x / gridDim.x;
   const int64_t i1 = a.nitems * (blockIdx.x + 1) / gridDim.x;
   const int nit = (int)(i1 - i0);
-  const int ntp = (int)a.ntp;
+  const int ntp = (int)a.ntp, nitf = (int)a.nit, T = a.tiles;
 
   if (tid == 0) {
     for (int i = 0; i < a.nst; ++i) {
       mbar_init(smem_u32(&hdr->full[i]), 1);
       mbar_init(smem_u32(&hdr->empty[i]), 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kAcc; ++i) {
       mbar_init(smem_u32(&hdr->accfull[i]), 1);
       mbar_init(smem_u32(&hdr->accempty[i]), kEpiThreads);
     }
@@ -198,8 +213,8 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
     int issued = 0, seg = 0, segs_loaded = 0;
     int fcur = -1;
     Cursor cu;
-    cu.init(i0, ntp, a.f0);
-    for (int i = 0; i < nit; ++i, cu.next(ntp, a.nst)) {
+    cu.init(i0, nitf, a.f0);
+    for (int i = 0; i < nit; ++i, cu.next(nitf, a.nst)) {
       const int f = cu.f, tp = cu.tp;
       if (f != fcur) {
         // the MMAs of the previous frequency must be done with B before it is replaced
@@ -218,10 +233,10 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
       const uint32_t fb = smem_u32(&hdr->full[s]);
       mbar_arrive_expect_tx(fb, stage_bytes);
       uint8_t* st = stages + (size_t)s * stage_bytes;
-      const int kb = 2 * (tp + (int)a.qtile0);
-      // one copy per operand: the tile's two 64-point blocks side by side
+      const int kb = 2 * (tp * T + (int)a.qtile0);
+      // one copy per operand: the item's 64-point blocks side by side
       tma_load_4d(smem_u32(st), &map_hi, 0, 0, f, kb, fb);
-      if (X3) tma_load_4d(smem_u32(st + 2 * a.box_bytes), &map_lo, 0, 0, f, kb, fb);
+      if (X3) tma_load_4d(smem_u32(st + op_bytes), &map_lo, 0, 0, f, kb, fb);
       issued = i + 1;
     }
     // copies still in flight must land before the CTA can exit
@@ -237,8 +252,8 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
     int seg = 0;
     int fcur = -1;
     Cursor cu;
-    cu.init(i0, ntp, a.f0);
-    for (int i = 0; i < nit; ++i, cu.next(ntp, a.nst)) {
+    cu.init(i0, nitf, a.f0);
+    for (int i = 0; i < nit; ++i, cu.next(nitf, a.nst)) {
       const int f = cu.f;
       if (f != fcur) {
         if (seg >= 1) mma_commit(smem_u32(&hdr->bempty));   // B of the previous frequency is released
@@ -246,24 +261,29 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
         fcur = f;
         ++seg;
       }
-      const int acc = i & 1;
-      if (i >= 2 && !mbar_wait(smem_u32(&hdr->accempty[acc]), ((i >> 1) - 1) & 1, abort_flag, gflags)) break;
       const int s = cu.s;
       if (!mbar_wait(smem_u32(&hdr->full[s]), cu.ph, abort_flag, gflags)) break;
       tc_fence_after();
       const uint32_t st = smem_u32(stages + (size_t)s * stage_bytes);
-      const uint32_t d = tmem + (uint32_t)acc * 128u;
-      for (int j = 0; j < nk16; ++j) {
-        // A: 16 K rows of both point boxes (MN atoms box_bytes apart); B: 16 K columns
-        const uint64_t da = sdesc_sw128(st + (uint32_t)j * 2048u, a.box_bytes, 1024);
-        const uint32_t boff = (uint32_t)(j >> 2) * katom_bytes + (uint32_t)(j & 3) * 32u;
-        const uint64_t db = sdesc_sw128(bhi + boff, 16, 1024);
-        mma_bf16(d, da, db, idesc, j > 0 ? 1u : 0u);
-        if (X3) {
-          const uint64_t dal = sdesc_sw128(st + 2 * a.box_bytes + (uint32_t)j * 2048u, a.box_bytes, 1024);
-          const uint64_t dbl = sdesc_sw128(blo + boff, 16, 1024);
-          mma_bf16(d, da, dbl, idesc, 1u);
-          mma_bf16(d, dal, db, idesc, 1u);
+      const int acc = i % kAcc;
+      if (i >= kAcc && !mbar_wait(smem_u32(&hdr->accempty[acc]), (i / kAcc - 1) & 1, abort_flag, gflags)) break;
+      tc_fence_after();
+      const int nv = min(T, ntp - cu.tp * T);
+      for (int t = 0; t < nv; ++t) {
+        const uint32_t d = tmem + (uint32_t)(acc * 128 + t * a.nn);
+        const uint32_t ta = st + (uint32_t)t * tile_bytes;
+        for (int j = 0; j < nk16; ++j) {
+          // A: 16 K rows of both point boxes (MN atoms box_bytes apart); B: 16 K columns
+          const uint64_t da = sdesc_sw128(ta + (uint32_t)j * 2048u, a.box_bytes, 1024);
+          const uint32_t boff = (uint32_t)(j >> 2) * katom_bytes + (uint32_t)(j & 3) * 32u;
+          const uint64_t db = sdesc_sw128(bhi + boff, 16, 1024);
+          mma_bf16(d, da, db, idesc, j > 0 ? 1u : 0u);
+          if (X3) {
+            const uint64_t dal = sdesc_sw128(ta + op_bytes + (uint32_t)j * 2048u, a.box_bytes, 1024);
+            const uint64_t dbl = sdesc_sw128(blo + boff, 16, 1024);
+            mma_bf16(d, da, dbl, idesc, 1u);
+            mma_bf16(d, dal, db, idesc, 1u);
+          }
         }
       }
       mma_commit(smem_u32(&hdr->empty[s]));
@@ -272,41 +292,62 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
     mma_commit(smem_u32(&hdr->drain));
     mbar_drain(smem_u32(&hdr->drain), 0, gflags);
   } else if (warp < kEpiWarps) {
-    // ---------------- epilogue: TMEM -> registers -> scaled complex stores
-    const int quad = warp & 3;
-    const int half = warp >> 2;
-    const int hcols = a.nn / 2;                     // columns of this warp: [half * hcols, +hcols)
-    const int k0 = half * (hcols / 2);              // first mode of this warp
+    // ---------------- epilogue: TMEM -> registers -> scaled complex stores.
+    // Groups of four warps (one per lane quadrant) take the CTA's items in turn;
+    // a warp takes all columns of its 32 points of every tile of the item.
+    const int quad = warp & 3, grp = warp >> 2;
     const int nm = a.nmodes;
-    Cursor cu;
-    cu.init(i0, ntp, a.f0);
-    for (int i = 0; i < nit; ++i, cu.next(ntp, a.nst)) {
-      const int f = cu.f, tp = cu.tp;
-      const int acc = i & 1;
-      // the point's output scale, requested before the wait for the
-      // accumulator so that its latency overlaps the item's copies and MMAs
-      const int64_t lm = tp * 128 + quad * 32 + lane;
-      const bool inrange = lm < a.mcount;
-      const float rw = inrange ? scale[a.m0 + lm] : 0.f;
+    const int plane = quad * 32 + lane;                // point of the tile
+    auto load_scale = [&](int tile) {
+      const int64_t lm = (int64_t)tile * 128 + plane;
+      return lm < a.mcount ? scale[a.m0 + lm] : 0.f;
+    };
+    int f = a.f0 + (int)(i0 / a.nit), tp = (int)(i0 % a.nit);
+    auto advance = [&](int n) {
+      tp += n;
+      while (tp >= nitf) { tp -= nitf; ++f; }
+    };
+    advance(grp);
+    float rw = grp < nit ? load_scale(tp * T) : 0.f;
+    for (int i = grp; i < nit; i += kEpiGroups) {
+      const int acc = i % kAcc;
+      const int tile0 = tp * T, nv = min(T, ntp - tile0);
+      float2* const of = phi + (int64_t)f * nm * a.M + (a.m0 - a.phioff);
+      advance(kEpiGroups);
       // one decision per warp: the tcgen05.ld below must be executed by the whole warp
-      const bool got = mbar_wait(smem_u32(&hdr->accfull[acc]), (i >> 1) & 1, abort_flag, gflags);
+      const bool got = mbar_wait(smem_u32(&hdr->accfull[acc]), (i / kAcc) & 1, abort_flag, gflags);
       if (!__all_sync(0xffffffffu, got)) break;
       tc_fence_after();
-      const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * 128u + (uint32_t)(half * hcols);
-      float v[64];
+      for (int t = 0; t < nv; ++t) {
+        const int64_t lm = (int64_t)(tile0 + t) * 128 + plane;
+        const bool inrange = lm < a.mcount;
+        const bool last = t + 1 == nv;
+        // the next tile's output scale: its latency overlaps this tile's work
+        const float rw_next = !last ? load_scale(tile0 + t + 1)
+                              : i + kEpiGroups < nit ? load_scale(tp * T) : 0.f;
+        uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 128 + t * a.nn);
+        float2* out = of + lm;
+        for (int c0 = 0; c0 < 2 * nm; c0 += 32) {      // 16 modes at a time
+          float v[32];
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
-        if (c * 8 < hcols) tmem_ld8(taddr + (uint32_t)(c * 8), v + c * 8);
-      tmem_wait_ld();
-      tc_fence_before();
-      mbar_arrive(smem_u32(&hdr->accempty[acc]));
-      if (inrange) {
-        const int64_t m = a.m0 + lm;
-        float2* out = phi + ((int64_t)f * nm + k0) * a.M + (m - a.phioff);
+          for (int c = 0; c < 4; ++c)
+            if (c0 + c * 8 < 2 * nm) tmem_ld8(taddr + (uint32_t)(c0 + c * 8), v + c * 8);
+          tmem_wait_ld();
+          if (last && c0 + 32 >= 2 * nm) {
+            tc_fence_before();
+            mbar_arrive(smem_u32(&hdr->accempty[acc]));
+          }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          if (2 * j < hcols && k0 + j < nm) out[(int64_t)j * a.M] = make_float2(v[2 * j] * rw, v[2 * j + 1] * rw);
+          for (int c = 0; c < 4; ++c)
+            if (c0 + c * 8 < 2 * nm) {                 // four modes
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                if (inrange && c0 / 2 + c * 4 + j < nm) *out = make_float2(v[8 * c + 2 * j] * rw, v[8 * c + 2 * j + 1] * rw);
+                out += a.M;
+              }
+            }
         }
+        rw = rw_next;
       }
     }
   }
@@ -322,18 +363,27 @@ int modes_np(const spod_plan_s& p) { return (2 * p.nb + 15) / 16 * 16; }
 int modes_nn(int nmodes) { return (2 * nmodes + 15) / 16 * 16; }
 uint32_t modes_img_bytes(int np, int nn) { return (uint32_t)((np + 63) / 64) * (uint32_t)nn * 128u; }
 
-size_t modes_tc_smem_stages(const spod_plan_s& p, int nst) {
+// 128-point tiles per item: a stage of about kStageTarget bytes.  One tile of
+// 16 rows (nb = 7) is 8 KB of hi and lo; with one tile per item and four
+// stages 32 KB were in flight per SM and every tile cost a hand-over.
+// An item's tiles share one accumulator buffer of 128 columns and one hand-over.
+int modes_tiles(const spod_plan_s& p, int nn) {
+  const int nops = p.desc.precision == SPOD_PREC_BF16X3 ? 2 : 1;
+  return std::max(1, std::min({kMaxTiles, kStageTarget / (2 * modes_np(p) * 128 * nops), 128 / nn}));
+}
+
+size_t modes_tc_smem_stages(const spod_plan_s& p, int nst, int tiles) {
   const int nops = p.desc.precision == SPOD_PREC_BF16X3 ? 2 : 1;
   const int np = modes_np(p);
   const size_t img = modes_img_bytes(np, modes_nn(std::max(p.nb, p.adj_cols)));   // the adjoint's extra column
   const size_t box = (size_t)np * 128;
-  return 1024 + 1024 + nops * img + (size_t)nst * 2 * box * nops;
+  return 1024 + 1024 + nops * img + (size_t)nst * tiles * 2 * box * nops;
 }
 
 }  // namespace
 
-// Shared memory of the smallest (2-stage) configuration; launches use up to 4 stages.
-size_t modes_tc_smem_bytes(const spod_plan_s& p) { return modes_tc_smem_stages(p, 2); }
+// Shared memory of the smallest (2-stage) configuration; launches use up to kMaxStages.
+size_t modes_tc_smem_bytes(const spod_plan_s& p) { return modes_tc_smem_stages(p, 2, 1); }
 
 // Per-frequency B images (hi [, lo]) for nmodes columns, in the plan's image buffer.
 size_t modes_image_bytes(const spod_plan_s& p) {
@@ -370,7 +420,9 @@ cudaError_t launch_modes_tc_chunk(const spod_plan_s& p, int64_t m0, int64_t mcou
   a.phioff = out_ld ? out_off : adjoint ? 0 : p.phi_off;
   a.ntp = (mcount + 127) / 128;
   a.qtile0 = qoff / 128;
-  a.nitems = a.ntp * (f1 - f0);
+  a.tiles = modes_tiles(p, a.nn);
+  a.nit = (a.ntp + a.tiles - 1) / a.tiles;
+  a.nitems = a.nit * (f1 - f0);
   a.f0 = f0;
   a.box_bytes = (uint32_t)a.np * 128u;
   a.img_bytes = modes_img_bytes(a.np, a.nn);
@@ -381,18 +433,23 @@ cudaError_t launch_modes_tc_chunk(const spod_plan_s& p, int64_t m0, int64_t mcou
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p.device);
   a.nst = kMaxStages;
-  while (a.nst > 2 && modes_tc_smem_stages(p, a.nst) > (size_t)optin) --a.nst;
-  const size_t smem = modes_tc_smem_stages(p, a.nst);
+  while (a.nst > 2 && modes_tc_smem_stages(p, a.nst, a.tiles) > (size_t)optin) --a.nst;
+  const size_t smem = modes_tc_smem_stages(p, a.nst, a.tiles);
+  CUtensorMap mh, ml;
+  const int64_t nblk = p.chunk_points / kQBlock;
+  if (!make_qhat_map(p, p.d_qhat, 2 * a.tiles, nblk, &mh) ||
+      !make_qhat_map(p, p.d_qlo ? p.d_qlo : p.d_qhat, 2 * a.tiles, nblk, &ml))
+    return cudaErrorUnknown;
   if (p.desc.precision == SPOD_PREC_BF16X3) {
     cudaError_t e = cudaFuncSetAttribute(k_modes_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_modes_tc<true><<<(unsigned)grid, kThreadsModes, smem, s>>>(p.tmap_hi2, p.tmap_lo2, a,
+    k_modes_tc<true><<<(unsigned)grid, kThreadsModes, smem, s>>>(mh, ml, a,
                                                                  static_cast<const uint8_t*>(p.d_bimg), scale,
                                                                  static_cast<float2*>(d_Phi), p.d_flags);
   } else {
     cudaError_t e = cudaFuncSetAttribute(k_modes_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_modes_tc<false><<<(unsigned)grid, kThreadsModes, smem, s>>>(p.tmap_hi2, p.tmap_hi2, a,
+    k_modes_tc<false><<<(unsigned)grid, kThreadsModes, smem, s>>>(mh, mh, a,
                                                                   static_cast<const uint8_t*>(p.d_bimg), scale,
                                                                   static_cast<float2*>(d_Phi), p.d_flags);
   }

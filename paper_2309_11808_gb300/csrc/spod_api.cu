@@ -208,32 +208,25 @@ void make_fft_store_maps(spod_plan_s* p) {
   p->fst_maps = true;
 }
 
-// TMA maps of the BF16 Qhat planes: dims {64 points, 2 nb rows, nf, chunk / 64},
-// box {64 points, 2 nb rounded up to 16 rows, 1, 1}; 128-byte swizzle.
-spod_status make_qhat_maps(spod_plan_s* p) {
-  auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p->encode_fn);
-  if (!encode) return fail(SPOD_ECUDA, "cuTensorMapEncodeTiled not available from the driver");
-  // blocked layout [chunk / 64][nf][2 nb][64] (qhat_blocked_offset): one box =
-  // one frequency's rows over one 64-point K step; rows past 2 nb read as zero
-  const cuuint64_t dims[4] = {(cuuint64_t)kQBlock, (cuuint64_t)p->qrows, (cuuint64_t)p->nf,
-                              (cuuint64_t)(p->chunk_points / kQBlock)};
+}  // namespace
+
+// TMA map of a BF16 Qhat plane in the blocked layout [chunk / 64][nf][qrows][64]
+// (qhat_blocked_offset): one box = one frequency's rows (2 nb rounded up to 16;
+// rows past qrows read as zero) over nbox consecutive 64-point blocks, 128-byte
+// swizzle; blocks from nblocks on read as zero.
+bool make_qhat_map(const spod_plan_s& p, void* base, int nbox, int64_t nblocks, CUtensorMap* map) {
+  auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p.encode_fn);
+  if (!encode) return false;
+  const cuuint64_t dims[4] = {(cuuint64_t)kQBlock, (cuuint64_t)p.qrows, (cuuint64_t)p.nf, (cuuint64_t)nblocks};
   const cuuint64_t row = (cuuint64_t)kQBlock * 2;
-  const cuuint64_t strides[3] = {row, row * p->qrows, row * p->qrows * p->nf};
+  const cuuint64_t strides[3] = {row, row * p.qrows, row * p.qrows * p.nf};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
-  void* bases[2] = {p->d_qhat, p->d_qlo ? p->d_qlo : p->d_qhat};
-  CUtensorMap* maps[4] = {&p->tmap_hi, &p->tmap_lo, &p->tmap_hi2, &p->tmap_lo2};
-  for (int i = 0; i < 4; ++i) {
-    // boxes of one 64-point block, and of two consecutive blocks (fewer, larger copies)
-    const cuuint32_t box[4] = {(cuuint32_t)kQBlock, (cuuint32_t)((2 * p->nb + 15) / 16 * 16), 1, i < 2 ? 1u : 2u};
-    CUresult r = encode(maps[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, bases[i & 1], dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(SPOD_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
-  }
-  return SPOD_OK;
+  const cuuint32_t box[4] = {(cuuint32_t)kQBlock, (cuuint32_t)((2 * p.nb + 15) / 16 * 16), 1, (cuuint32_t)nbox};
+  return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-}  // namespace
 }  // namespace spod
 
 using namespace spod;
@@ -483,11 +476,9 @@ spod_status spod_plan_create(const spod_plan_desc* d, spod_plan_t* out) {
   p->ring_ok = p->pipe_ok || (!p->cplx && p->encode_fn &&
                               fft_ring_usable(*p, (int)prop.sharedMemPerBlockOptin));
   if (p->tensor) {
-    if (spod_status st = make_qhat_maps(p)) {
-      std::string msg = spod_last_error();
-      spod_plan_destroy(p);
-      return fail(st, msg);
-    }
+    CUtensorMap probe;               // the kernels' launches encode their own
+    if (!make_qhat_map(*p, p->d_qhat, 2, p->chunk_points / kQBlock, &probe))
+      return bail(SPOD_ECUDA, "cuTensorMapEncodeTiled (Qhat) failed or not available from the driver");
   }
 
   // ---- constant tables (host FP64, rounded once to the compute type)

@@ -110,10 +110,6 @@ struct spod_plan_s {
   void* d_qhat = nullptr;          // [nf][2*nb][chunk_points] compute type (planar re | im); BF16 hi for tensor precisions
   void* d_qlo = nullptr;           // BF16X3: the lo part, same layout
   bool tensor = false;             // BF16 / BF16X3: Gram and modes on the tensor cores
-  CUtensorMap tmap_hi;            // TMA maps of d_qhat / d_qlo: dims {chunk, 2nb, nf}, box {64, round16(2nb), 1}
-  CUtensorMap tmap_lo;
-  CUtensorMap tmap_hi2;           // the same planes, box {64, round16(2nb), 1, 2}: two 64-point blocks per copy
-  CUtensorMap tmap_lo2;
   CUtensorMap tmap_fst_hi;         // FFT output store maps: dims {chunk, 2nb, nf}, box {16, 1, 256}
   CUtensorMap tmap_fst_lo;         //   (FP32 planes, or BF16 hi / lo)
   bool fst_maps = false;
@@ -194,6 +190,7 @@ cudaError_t launch_adjoint_chunk(const spod_plan_s& p, const void* d_R, int64_t 
                                  int64_t mcount, void* d_dX, cudaStream_t s);
 size_t adjoint_smem_bytes(const spod_plan_s& p);
 
+bool make_qhat_map(const spod_plan_s& p, void* base, int nbox, int64_t nblocks, CUtensorMap* map);
 cudaError_t launch_gram_tc_chunk(const spod_plan_s& p, int64_t mcount, bool first, cudaStream_t s);
 cudaError_t launch_modes_tc_chunk(const spod_plan_s& p, int64_t m0, int64_t mcount, int nmodes, void* d_Phi,
                                   cudaStream_t s, bool adjoint = false, int f0 = 0, int f1 = -1, int64_t qoff = 0,
