@@ -359,11 +359,12 @@ typedef struct {
                              plans) leaves its first pipeline stage unfilled, so the waits on it run
                              out after wait_timeout_us and the fit reports SPOD_ETIMEOUT; 0 (default):
                              off.  No other effect. */
-  int fft_tile_points;    /* pipelined FFT (compiled nfft): spatial points per CTA tile, 16 (two CTAs
-                             per SM up to nfft 512) or 32 (one CTA per SM, whole 128-byte rows); the
-                             plan picks 32 where it fits in shared memory.  0 on read: the plan does
-                             not use the pipelined FFT; 0 on write: leave as is.  Changes only the
-                             launch shape, not the results. */
+  int fft_tile_points;    /* pipelined FFT (compiled nfft): spatial points per CTA tile, 16, or 32 for
+                             the widest form the plan has (32 points; 64 where it measured faster),
+                             narrowed for grids with fewer such tiles than SMs; the plan picks 32
+                             where it fits in shared memory.  0 on read: the plan does not use the
+                             pipelined FFT; 0 on write: leave as is.  Changes only the launch shape,
+                             not the results. */
 } spod_tuning;
 
 /* The plan's launch shape into *tuning (host).  No counterpart in the paper. */

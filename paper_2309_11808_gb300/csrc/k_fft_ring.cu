@@ -1,5 +1,5 @@
 // Persistent block DFT (Eqs. blocks, blocks-ft, blocks-k) with a TMA ring, for
-// nfft values without a compiled radix sequence (those use k_fft_pipe.cu).
+// nfft values without a compiled radix sequence (those use fft_pipe.cuh).
 //
 // Persistent CTAs of 512 threads walk tiles of 16 spatial points; for each tile
 // a CTA transforms the Welch blocks l = 0 .. nb-1 in order.  The tile's time
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(RTHREADS, 1) k_fft_ring(const __grid_constant_
                                                           unsigned* __restrict__ gflags) {
   using namespace tc;
   extern __shared__ unsigned char smem_raw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sm = smem_align1024(smem_raw);
   RingHdr* hdr = reinterpret_cast<RingHdr*>(sm);
   Tin* ring = reinterpret_cast<Tin*>(sm + 1024);                        // [ring rows][RTP]
   float2* buf = reinterpret_cast<float2*>(sm + 1024 + (size_t)a.ring * RTP * sizeof(Tin));

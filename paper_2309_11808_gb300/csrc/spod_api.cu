@@ -139,8 +139,17 @@ void* driver_encode_fn() {
   return fn;
 }
 
-// TMA map of X for the ring FFTs: dims {M, nt}, box {tile points, ring_boxr rows}.
-spod_status make_x_map(const spod_plan_s* p, const void* d_X, CUtensorMap* map) {
+// X for the TMA-fed FFT kernels: its map, dims {M, nt}, box {tile points,
+// ring_boxr rows}, and the tile width.
+struct XMap {
+  alignas(64) CUtensorMap map;
+  int width = 16;
+};
+
+// The map for FFT launches over (at most) `points` points each.
+spod_status make_x_map(const spod_plan_s* p, const void* d_X, int64_t points, XMap* xm) {
+  CUtensorMap* const map = &xm->map;
+  if (p->pipe_ok) xm->width = fft_pipe_width(*p, points);
   auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p->encode_fn);
   if (!encode) return fail(SPOD_ECUDA, "cuTensorMapEncodeTiled not available");
   // complex data: a [nt][2M] array of interleaved real components
@@ -153,7 +162,7 @@ spod_status make_x_map(const spod_plan_s* p, const void* d_X, CUtensorMap* map) 
                                                                   : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)p->nt};
   const cuuint64_t strides[1] = {(cuuint64_t)cols * el};
-  const cuuint32_t box[2] = {(cuuint32_t)(p->pipe_ok ? p->pipe_tp : 16), (cuuint32_t)p->ring_boxr};
+  const cuuint32_t box[2] = {(cuuint32_t)xm->width, (cuuint32_t)p->ring_boxr};
   const cuuint32_t estr[2] = {1, 1};
   CUresult r = encode(map, dt, 2, const_cast<void*>(d_X), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                       CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -162,14 +171,15 @@ spod_status make_x_map(const spod_plan_s* p, const void* d_X, CUtensorMap* map) 
 }
 
 // FFT of one spatial chunk: the TMA-ring kernel when the shape allows it.
-spod_status run_fft_chunk(spod_plan_s* p, const void* d_X, const CUtensorMap* xmap, int64_t m0, int64_t mc,
-                          cudaStream_t s) {
+spod_status run_fft_chunk(spod_plan_s* p, const void* d_X, const XMap* xmap, int64_t m0, int64_t mc,
+                          cudaStream_t s, int* nlaunch) {
   // the folded mean lives in the pipelined kernel only (mean_fold implies pipe_ok,
   // and every caller builds the X map when ring_ok holds)
   if (p->mean_fold && !xmap) return fail(SPOD_EUNSUPPORTED, "folded time mean without the X tensor map");
+  if (!xmap || !p->pipe_ok) ++*nlaunch;
   cudaError_t e = !xmap        ? launch_fft_chunk(*p, d_X, m0, mc, s)
-                  : p->pipe_ok ? launch_fft_pipe_chunk(*p, *xmap, d_X, m0, mc, s)
-                               : launch_fft_ring_chunk(*p, *xmap, m0, mc, s);
+                  : p->pipe_ok ? launch_fft_pipe_chunk(*p, xmap->map, xmap->width, d_X, m0, mc, s, nlaunch)
+                               : launch_fft_ring_chunk(*p, xmap->map, m0, mc, s);
   if (e != cudaSuccess) return cuda_fail(e, "fft kernel");
   return SPOD_OK;
 }
@@ -360,8 +370,8 @@ spod_status spod_plan_create(const spod_plan_desc* d, spod_plan_t* out) {
   // ---- which FFT kernel; whether the time mean is folded into it
   {
     const bool q = p->encode_fn != nullptr;
-    if (q) p->pipe_tp = fft_pipe_tile(*p, (int)prop.sharedMemPerBlockOptin);
-    p->pipe_ok = q && fft_pipe_usable(*p, (int)prop.sharedMemPerBlockOptin);
+    if (q) p->pipe_tp = fft_pipe_tile(*p);
+    p->pipe_ok = q && prop.sharedMemPerBlockOptin >= 227 * 1024 && fft_pipe_usable(*p);
   }
   p->mean_fold = d->mean_in_fft && p->tensor && p->pipe_ok && !p->cplx && d->subtract_mean &&
                  (2 * p->nb + 1 + 15) / 16 == (2 * p->nb + 15) / 16;
@@ -606,10 +616,10 @@ static spod_status fit_impl(spod_plan_t p, const void* d_X, cudaStream_t s, int6
   SPOD_CUDA(cudaMemsetAsync(p->d_flags, 0, sizeof(unsigned), s), "clear flags");   // [1] is the wait bound
   if (!p->desc.subtract_mean)
     SPOD_CUDA(cudaMemsetAsync(p->d_mu, 0, sizeof(double) * p->M * (p->cplx ? 2 : 1), s), "zero mean");
-  alignas(64) CUtensorMap xmap;
-  const CUtensorMap* xm = nullptr;
+  XMap xmap;
+  const XMap* xm = nullptr;
   if (p->ring_ok) {
-    if (spod_status st = make_x_map(p, d_X, &xmap)) return st;
+    if (spod_status st = make_x_map(p, d_X, std::min<int64_t>(w, p->M), &xmap)) return st;
     xm = &xmap;
   }
   int64_t nchunks = 0;
@@ -620,8 +630,8 @@ static spod_status fit_impl(spod_plan_t p, const void* d_X, cudaStream_t s, int6
       SPOD_CUDA(launch_mean(*p, d_X, m0, mc, s), "mean kernel");
     }
     {
-      Phase ph(p, SPOD_PHASE_FFT, s, 1);
-      if (spod_status st = run_fft_chunk(p, d_X, xm, m0, mc, s)) return st;
+      Phase ph(p, SPOD_PHASE_FFT, s, 0);
+      if (spod_status st = run_fft_chunk(p, d_X, xm, m0, mc, s, &ph.n)) return st;
     }
     Phase ph(p, SPOD_PHASE_GRAM, s, p->tensor ? 2 : 1);
     if (p->tensor) SPOD_CUDA(launch_gram_tc_chunk(*p, mc, m0 == 0, s), "tensor-core gram kernel");
@@ -759,17 +769,17 @@ static spod_status modes_impl(spod_plan_t p, const void* d_X, int nmodes, void* 
       if (done) SPOD_CUDA(cudaEventRecord(done[r], s), "range done");
     }
   } else {
-    alignas(64) CUtensorMap xmap;
-    const CUtensorMap* xm = nullptr;
+    XMap xmap;
+    const XMap* xm = nullptr;
     if (p->ring_ok) {
-      if (spod_status st = make_x_map(p, d_X, &xmap)) return st;
+      if (spod_status st = make_x_map(p, d_X, std::min<int64_t>(p->chunk_points, p->M), &xmap)) return st;
       xm = &xmap;
     }
     for (int64_t m0 = 0; m0 < p->M; m0 += p->chunk_points) {
       const int64_t mc = std::min<int64_t>(p->chunk_points, p->M - m0);
       {
-        Phase ph(p, SPOD_PHASE_FFT, s, 1);
-        if (spod_status st = run_fft_chunk(p, d_X, xm, m0, mc, s)) return st;
+        Phase ph(p, SPOD_PHASE_FFT, s, 0);
+        if (spod_status st = run_fft_chunk(p, d_X, xm, m0, mc, s, &ph.n)) return st;
       }
       Phase ph(p, SPOD_PHASE_MODES, s, 0);
       if (p->tensor) {
@@ -816,10 +826,10 @@ spod_status spod_backward(spod_plan_t p, const double* d_dLdlambda, const void* 
     SPOD_CUDA(launch_mode_image(*p, p->adj_cols, s), "adjoint operand image kernel");
     ph.n += 1;
   }
-  alignas(64) CUtensorMap xmap;
-  const CUtensorMap* xm = nullptr;
+  XMap xmap;
+  const XMap* xm = nullptr;
   if (!p->qhat_valid && p->ring_ok) {
-    if (spod_status st = make_x_map(p, d_X, &xmap)) return st;
+    if (spod_status st = make_x_map(p, d_X, std::min<int64_t>(p->chunk_points, p->M), &xmap)) return st;
     xm = &xmap;
   }
   // per Qhat chunk (recomputed unless the fit left it in place), per column
@@ -830,8 +840,7 @@ spod_status spod_backward(spod_plan_t p, const double* d_dLdlambda, const void* 
   for (int64_t m0 = 0; m0 < p->M; m0 += p->chunk_points) {
     const int64_t mc = std::min<int64_t>(p->chunk_points, p->M - m0);
     if (!p->qhat_valid) {
-      if (spod_status st = run_fft_chunk(p, d_X, xm, m0, mc, s)) return st;
-      ph.n += 1;
+      if (spod_status st = run_fft_chunk(p, d_X, xm, m0, mc, s, &ph.n)) return st;
     }
     for (int64_t s0 = m0; s0 < m0 + mc; s0 += rw) {
       const int64_t sw = std::min<int64_t>(rw, m0 + mc - s0);
@@ -1078,20 +1087,20 @@ spod_status spod_run_host_ooc(spod_plan_t p, const void* h_X, int nmodes, void* 
   p->x_ld = w;
   ck(cudaMemsetAsync(p->d_flags, 0, sizeof(unsigned), s), "clear flags");      // [1] is the wait bound
   if (!p->desc.subtract_mean) ck(cudaMemsetAsync(p->d_mu, 0, sizeof(double) * M * (p->cplx ? 2 : 1), s), "zero mean");
-  int use = 0;
+  int use = 0, nl = 0;
   for (int64_t c = 0; c < ntile && st == SPOD_OK; ++c, ++use) {
     const int b = use & 1;
     const int64_t c0 = c * w, wc = std::min<int64_t>(w, M - c0);
     gather(c, b, use);
     p->x_off = c0;
     if (p->desc.subtract_mean && !p->mean_fold) ck(launch_mean(*p, xt[b], c0, wc, s), "mean kernel");
-    alignas(64) CUtensorMap xmap;
-    const CUtensorMap* xm = nullptr;
+    XMap xmap;
+    const XMap* xm = nullptr;
     if (p->ring_ok && st == SPOD_OK) {
-      if ((st = make_x_map(p, xt[b], &xmap)) != SPOD_OK) break;
+      if ((st = make_x_map(p, xt[b], w, &xmap)) != SPOD_OK) break;
       xm = &xmap;
     }
-    if (st == SPOD_OK) st = run_fft_chunk(p, xt[b], xm, c0, wc, s);
+    if (st == SPOD_OK) st = run_fft_chunk(p, xt[b], xm, c0, wc, s, &nl);
     if (p->tensor) ck(launch_gram_tc_chunk(*p, wc, c == 0, s), "tensor-core gram kernel");
     else ck(launch_gram_chunk(*p, wc, c == 0, s), "gram kernel");
     ck(cudaEventRecord(xfree[b], s), "event");
@@ -1116,17 +1125,16 @@ spod_status spod_run_host_ooc(spod_plan_t p, const void* h_X, int nmodes, void* 
       const int64_t c0 = c * w, wc = std::min<int64_t>(w, M - c0);
       gather(c, b, use);
       p->x_off = c0;
-      alignas(64) CUtensorMap xmap;
-      const CUtensorMap* xm = nullptr;
+      XMap xmap;
+      const XMap* xm = nullptr;
       if (p->ring_ok) {
-        if ((st = make_x_map(p, xt[b], &xmap)) != SPOD_OK) break;
+        if ((st = make_x_map(p, xt[b], w, &xmap)) != SPOD_OK) break;
         xm = &xmap;
       }
-      if ((st = run_fft_chunk(p, xt[b], xm, c0, wc, s)) != SPOD_OK) break;
+      if ((st = run_fft_chunk(p, xt[b], xm, c0, wc, s, &nl)) != SPOD_OK) break;
       ck(cudaEventRecord(xfree[b], s), "event");
       if (c >= 2) ck(cudaStreamWaitEvent(s, pfree[pb], 0), "wait");
       p->phi_off = c0;
-      int nl = 0;
       if (p->tensor) ck(launch_modes_tc_chunk(*p, c0, wc, nmodes, pt[pb], s), "tensor-core modes kernel");
       else ck(launch_modes_chunk(*p, c0, wc, nmodes, pt[pb], s, &nl), "modes kernel");
       ck(cudaEventRecord(pready[pb], s), "event");
@@ -1224,10 +1232,7 @@ spod_status spod_plan_set_tuning(spod_plan_t p, const spod_tuning* t) {
     if (!p->pipe_ok) return fail(SPOD_EINVAL, "fft_tile_points: this plan does not use the pipelined FFT");
     if (t->fft_tile_points != 16 && t->fft_tile_points != 32)
       return fail(SPOD_EINVAL, "fft_tile_points must be 16 or 32");
-    int optin = 0;
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
-    const size_t sm = fft_pipe_smem_bytes(*p, t->fft_tile_points);
-    if (sm == 0 || sm > (size_t)optin)
+    if (!fft_pipe_has(*p, t->fft_tile_points))
       return fail(SPOD_EINVAL, "fft_tile_points: no form of the pipelined FFT with that tile for this plan");
   }
   if (t->wait_timeout_us != p->wait_timeout_us) {
@@ -1402,12 +1407,8 @@ spod_status spod_plan_autotune(spod_plan_t p, const void* d_X, void* stream, spo
   // FFT tile widths with a compiled form that fits (pipelined FFT only)
   std::vector<int> tiles;
   if (p->pipe_ok) {
-    int optin = 0;
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
-    for (int tp : {16, 32}) {
-      const size_t sm = fft_pipe_smem_bytes(*p, tp);
-      if (sm > 0 && sm <= (size_t)optin) tiles.push_back(tp);
-    }
+    for (int tp : {16, 32})
+      if (fft_pipe_has(*p, tp)) tiles.push_back(tp);
   }
   const int keep_splits = p->gram_splits, keep_tp = p->pipe_tp;
   const int prof = p->prof;

@@ -32,7 +32,7 @@ constexpr int kEigSmemMaxNb = 48;      // eigen-solver keeps A and V in shared m
 // K step of one frequency is a single contiguous qrows x 128-byte box for the
 // tensor-core kernels.  Rows are re = l, im = nb + l for Welch block l; when
 // the time mean is folded into the FFT (spod_plan_s::mean_fold) one more row,
-// 2 nb, holds rho_m = sqrt(W_m) (mu_m - x_m(t = 0)) of every point (qrows =
+// 2 nb, holds rho_m = sqrt(W_m) (mu_m - c_m) of every point (c_m: the centre; qrows =
 // 2 nb + 1), the input of the rank-one mean correction of the consumers.
 constexpr int kQBlock = 64;
 __host__ __device__ inline int64_t qhat_blocked_offset(int nf, int qrows, int f, int row, int64_t m) {
@@ -94,7 +94,7 @@ struct spod_plan_s {
   // correction Qhat = Z - mu' What_f.  No separate mean pass reads X.
   bool mean_fold = false;
   int qrows = 0;              // Qhat rows per frequency: 2 nb (+ 1 with mean_fold)
-  int pipe_tp = 16;           // its tile width in points (16 or 32; also the X map's box width)
+  int pipe_tp = 16;           // its tile choice: 16 points, or 32 and wider (fft_pipe_width)
   void* encode_fn = nullptr;  // cuTensorMapEncodeTiled
   int num_sms = 0;
 
@@ -213,12 +213,23 @@ size_t fft_ring_smem_bytes(const spod_plan_s& p);
 size_t fft_ring_stage_offset(const spod_plan_s& p);
 size_t fft_ring_plane_elems(const spod_plan_s& p);
 bool fft_ring_usable(const spod_plan_s& p, int smem_optin);
-size_t fft_pipe_smem_bytes(const spod_plan_s& p, int tp);
-bool fft_pipe_usable(const spod_plan_s& p, int smem_optin);
-int fft_pipe_tile(const spod_plan_s& p, int smem_optin);
-cudaError_t launch_fft_pipe_chunk(const spod_plan_s& p, const CUtensorMap& xmap, const void* d_X, int64_t m0,
-                                  int64_t mcount,
-                                  cudaStream_t s);
+// The pipelined FFT of one compiled nfft (one translation unit each).
+struct PipeLen {
+  bool (*has)(const spod_plan_s& p, int tp) = nullptr;
+  int (*width)(const spod_plan_s& p, int64_t points) = nullptr;
+  cudaError_t (*launch)(const spod_plan_s& p, const CUtensorMap& xmap, int width, const void* d_X, int64_t m0,
+                        int64_t mcount, cudaStream_t s, int* nlaunch) = nullptr;
+};
+PipeLen pipe_len_256();
+PipeLen pipe_len_384();
+PipeLen pipe_len_512();
+PipeLen pipe_len_720();
+bool fft_pipe_has(const spod_plan_s& p, int tp);
+bool fft_pipe_usable(const spod_plan_s& p);
+int fft_pipe_tile(const spod_plan_s& p);
+int fft_pipe_width(const spod_plan_s& p, int64_t points);
+cudaError_t launch_fft_pipe_chunk(const spod_plan_s& p, const CUtensorMap& xmap, int width, const void* d_X, int64_t m0,
+                                  int64_t mcount, cudaStream_t s, int* nlaunch);
 cudaError_t launch_fft_ring_chunk(const spod_plan_s& p, const CUtensorMap& xmap, int64_t m0, int64_t mcount,
                                   cudaStream_t s);
 size_t eig_smem_bytes(int nb);

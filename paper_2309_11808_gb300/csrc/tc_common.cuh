@@ -24,6 +24,13 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// First 1024-byte boundary of a dynamic shared-memory array.  Pointer arithmetic
+// on the array itself (not an integer round trip), so that accesses through the
+// result stay shared-memory instructions and not generic ones.
+__device__ __forceinline__ uint8_t* smem_align1024(unsigned char* raw) {
+  return raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
+}
+
 __device__ __forceinline__ uint64_t globaltimer() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -105,6 +112,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same by a whole warp, with one decision for it.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                               unsigned* gflags) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, gflags));
+}
+
 // Bounded wait that ignores the CTA's abort flag: lets copies or MMAs already
 // in flight complete before the CTA releases their resources and exits.
 __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, unsigned* gflags) {
@@ -118,6 +131,19 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, unsign
   }
   return true;
 }
+
+// One lane of a converged warp (the same one at every call).  The issuing warps
+// run their loops as whole warps on warp-uniform values and leave only the
+// instruction itself to this lane: tcgen05.mma and TMA take their descriptors from
+// uniform registers, and a loop run by one lane (if (lane == 0)) had to move each
+// one there first, about 150 cycles per MMA.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// The warp's index, as a value that is the same in all its lanes.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 
 // ---------------------------------------------------------------- fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
