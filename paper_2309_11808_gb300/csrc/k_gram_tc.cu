@@ -5,20 +5,12 @@
 // Real embedding: with Y_f = [Re Qhat_f ; Im Qhat_f] (2nb rows x points, K-major
 // in HBM; sqrt(W) is already folded into Qhat), D = Y_f Y_f^T gives
 //   Re M_f[l][l'] = D[l][l'] + D[nb+l][nb+l'],  Im M_f[l][l'] = D[l][nb+l'] - D[nb+l][l'].
-// An item is kpb 64-point blocks of one frequency; its stage holds the TMA
-// boxes (NP rows x 64 points x kpb blocks, NP = 2nb rounded up to 16, 128-byte
-// swizzle) of hi and, for BF16X3, of lo.  The MMA always has M = 128 rows, so
-// with NP <= 64 it takes P = 128 / NP consecutive blocks of the stage at once
-// (their rows are contiguous): A = B = the P x NP stacked rows, N = P x NP, and
-// of D only the P diagonal NP x NP blocks are read, one A1 run per block each
-// as before (the same MMAs on the same rows, so the same rounding).  A stage,
-// an MMA group and a drain then cover P blocks: with 16 rows (nb = 7) a
-// 64-point block is 4 KB, and one hand-over per block left the kernel waiting
-// for its hand-overs: 361 x 720 x 2 points, 361 bins, nb = 7, bf16x3 took
-// 11.5 ms and takes 2.3 (4.8 TB/s of Qhat); with 48 rows (nb = 21, 193 bins)
-// 6.2 -> 3.5 ms.  Per K step of 16:
+// An item is up to KPB 64-point blocks of one frequency; its stage holds the TMA
+// boxes (NP rows x 64 points x KPB blocks, NP = 2nb rounded up to 16, 128-byte
+// swizzle) of hi and, for BF16X3, of lo.  Per K step of 16 (N = NP):
 //   A1 (+)= hi hi^T   restarted every `flush` blocks (short FP32 runs in the
-//                      tensor core), drained into Kahan-compensated registers.
+//                      tensor core, HB runs side by side in a tensor-memory
+//                      buffer), drained into Kahan-compensated registers.
 //                      The tensor core's FP32 accumulation rounds toward zero,
 //                      so a run of R MMAs carries a relative bias of about
 //                      R * 2^-24 on the positive diagonal; measured on the
@@ -36,8 +28,19 @@
 // 2.4e-6 of D) that would shift small eigenvalues.  A operand rows >= 2nb only
 // feed accumulator rows that are never read.
 //
+// What bounds it: the read of Qhat, as long as an item and a hand-over are large
+// enough.  With few Welch blocks a 64-point block is small (16 rows, nb = 7: 4 KB of
+// hi and lo) and one copy per two blocks and one hand-over per run left the kernel
+// waiting for them; so KPB and HB grow as NP shrinks, with the runs and the order
+// of the sums as before.  The issue of the MMAs came next: a loop run by one lane spent
+// about 150 cycles per MMA, so the MMA and TMA warps run as whole warps (elect_one),
+// and the warps that sum the lo squares load a block's rows in one batch.  bf16x3,
+// 361 x 720 x 2 points: nb = 7, 361 bins 11.5 -> 4.1 ms (now 55 cycles per N = 16 MMA
+// bound it), nb = 21, 193 bins 6.2 -> 3.0 (5.7 TB/s of Qhat); 512 x 256 x 3 points,
+// nb = 38, 257 bins 6.8 -> 5.0 (6.2 TB/s); BF16, nb = 33, 129 bins 4.2 -> 2.9.
+//
 // Persistent CTAs (one per SM by default) walk a contiguous range of the
-// f-major list of (frequency, block pair) items.  Warp 8 issues TMA into a
+// f-major list of (frequency, block pair) entries, up to KPB / 2 pairs an item.  Warp 8 issues TMA into a
 // ring of stages, warp 9 issues the MMAs, warps 0-7 drain TMEM (two warps per
 // lane quadrant, half of the columns each; quadrants without a row < 2nb
 // skip the reads) and warps 10-11 sum the lo squares.  When the CTA's run of
@@ -53,26 +56,28 @@ namespace spod {
 namespace {
 
 constexpr int kMaxStages = 8;
-// 64-point blocks per MMA (stacked diagonal blocks of D) for np rows per block
-__host__ __device__ constexpr int gram_pack(int np) { return np <= 64 ? 128 / np : 1; }
-// 64-point blocks per item (one TMA copy per operand): whole MMA packs, and at
-// least two blocks (with 80 rows, items of one block measured 6.88 ms against
-// 6.79 on the 512 x 256 x 3 grid)
-__host__ __device__ constexpr int gram_kpb(int np) { return gram_pack(np) > 2 ? gram_pack(np) : 2; }
+// 64-point blocks per item (one TMA copy per operand) for np rows: 16 to 24 KB per
+// operand where the rows are few (with 80 rows, items of one block measured
+// 6.88 ms against 6.79 on the 512 x 256 x 3 grid)
+__host__ __device__ constexpr int gram_kpb(int np) { return np <= 16 ? 8 : np <= 48 ? 4 : 2; }
+// A1 runs per tensor-memory buffer and hand-over: an item's, while two such buffers
+// and the two A2 buffers fit the 512 columns (np = 80: two runs a hand-over 5.0 ms
+// against 5.8 with one, 512 x 256 x 3 points, nb = 38, bf16x3)
+__host__ __device__ constexpr int gram_hb(int np) { return np <= 80 ? gram_kpb(np) : 1; }
 constexpr int kEpiWarps = 8;
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1, kDiagWarp0 = kEpiWarps + 2;
 constexpr int kDiagThreads = 64;
 constexpr int kThreadsGram = (kEpiWarps + 4) * 32;
-constexpr uint32_t kTmemCols = 512;       // A1 buffers at columns b * np (b < nacc), then two A2 buffers
+constexpr uint32_t kTmemCols = 512;       // A1 buffers at columns b * HB * np (b < nacc), then two A2 buffers
 constexpr int kMaxAcc = 4;                // A1 accumulator buffers at most
 
 struct GramTcArgs {
   int nb, r2, np, nf;
-  int64_t nkb;                            // items per frequency in this chunk
-  int64_t nsb;                            // packs of P 64-point blocks per frequency in this chunk
-  int64_t nitems;                         // nf * nkb
-  int flush;                              // packs (64-point blocks of one diagonal block) per A1 run
+  int64_t nkb;                            // block pairs per frequency in this chunk
+  int64_t nblk;                           // 64-point blocks per frequency in this chunk
+  int64_t nitems;                         // nf * nkb block pairs
+  int flush;                              // 64-point blocks per A1 run
   int nacc;                               // A1 buffers in tensor memory (2..kMaxAcc, as np allows)
   int stall0;                             // self-test: the first item's copies are never issued, so
                                           // every wait on them runs out (the bounded-wait path)
@@ -124,57 +129,81 @@ struct GramHdr {
   int abort;
 };
 
-// Walks the group and segment structure of a CTA's range, one pack (P
-// 64-point blocks) at a time: a segment is the run of one frequency, a group
-// (one A1 run in tensor memory) at most `flush` consecutive packs of a
-// segment; a group may end inside an item.  All roles step it identically.
+// Walks the run, group and segment structure of a CTA's range, one 64-point
+// block at a time: a segment is the part of one frequency, a run (one A1
+// accumulation) at most `flush` consecutive blocks of a segment, a group (the
+// runs of one tensor-memory buffer) at most HB consecutive runs; both may end
+// inside an item.  All roles step it identically.
+template <int HB>
 struct GroupWalk {
   int fprev = -1;
-  int in_group = 0;
+  int in_run = 0, run = 0;      // blocks of the current run so far; its place in the group
   int g = -1, seg = -1;
   int acc = -1, accph = 0;      // the group's A1 buffer and the parity of its use (g / nacc) & 1
-  bool sstart = false;
+  bool sstart = false, rstart = false;
   __device__ __forceinline__ bool step(int f, int flush, int nacc) {   // true when the block starts a group
     sstart = f != fprev;
-    const bool start = sstart || in_group == flush;
+    rstart = sstart || in_run == flush;
+    bool start = false;
     if (sstart) ++seg;
-    if (start) {
-      ++g;
-      in_group = 0;
-      if (++acc == nacc) { acc = 0; accph ^= 1; }
+    if (rstart) {
+      in_run = 0;
+      start = sstart || run + 1 == HB;
+      run = start ? 0 : run + 1;
+      if (start) {
+        ++g;
+        if (++acc == nacc) { acc = 0; accph ^= 1; }
+      }
     }
-    ++in_group;
+    ++in_run;
     fprev = f;
     return start;
   }
+  // an item that is a group of its own, a run per block
+  __device__ __forceinline__ void item(int f, int nacc) {
+    sstart = f != fprev;
+    if (sstart) ++seg;
+    ++g;
+    if (++acc == nacc) { acc = 0; accph ^= 1; }
+    fprev = f;
+  }
+  // whether the group ends with the current block (send: the segment does)
+  __device__ __forceinline__ bool ends(bool send, int flush) const {
+    return send || (in_run == flush && run + 1 == HB);
+  }
 };
 
-// Position of a CTA's item in the (frequency, block pair) list and in the
-// stage ring, advanced without divisions (the issuing threads are on the
+// Position of a CTA in the (frequency, block pair) list and in the stage ring, an
+// item at a time, advanced without divisions (the issuing threads are on the
 // critical path of every item).
+template <int KP>
 struct Cursor {
-  int f, kp;          // frequency, block pair within it
+  int f, kp;          // frequency, the item's first block pair within it
+  int left;           // the CTA's pairs from there on
+  int n;              // pairs of the item
   int s, ph;          // stage, parity of the ring pass (i / nst) & 1
-  __device__ __forceinline__ void init(int64_t item0, int nkb) {
-    f = (int)(item0 / nkb);
-    kp = (int)(item0 - (int64_t)f * nkb);
+  __device__ __forceinline__ void init(int64_t pair0, int npair, int nkb) {
+    f = (int)(pair0 / nkb);
+    kp = (int)(pair0 - (int64_t)f * nkb);
+    left = npair;
+    n = min(KP, min(nkb - kp, left));
     s = 0;
     ph = 0;
   }
-  __device__ __forceinline__ bool last_of_f(int nkb) const { return kp + 1 == nkb; }
+  __device__ __forceinline__ bool more() const { return left > 0; }
+  __device__ __forceinline__ bool seg_end(int nkb) const { return n == left || kp + n == nkb; }
   __device__ __forceinline__ void next(int nkb, int nst) {
-    if (++kp == nkb) { kp = 0; ++f; }
+    kp += n;
+    left -= n;
+    if (kp == nkb) { kp = 0; ++f; }
+    n = min(KP, min(nkb - kp, left));
     if (++s == nst) { s = 0; ph ^= 1; }
   }
 };
 
-// Slot of one (CTA, frequency): P sub-slots, one per diagonal block of D.
-// Sub-slot layout (bytes): A1 (sum, carry) pairs [r2][r2] float2, A2 [r2][r2]
-// float, then (sub-slot 0 only) the lo-square diagonal [r2] float; whole
-// 8-byte words, so that every sub-slot's pairs are aligned.
-__host__ __device__ inline size_t gram_slot_bytes(int r2) {
-  return ((size_t)r2 * r2 * 12 + (size_t)r2 * 4 + 7) / 8 * 8;
-}
+// Slot layout (bytes): A1 (sum, carry) pairs [r2][r2] float2, A2 [r2][r2]
+// float, then the lo-square diagonal [r2] float.
+__host__ __device__ inline size_t gram_slot_bytes(int r2) { return (size_t)r2 * r2 * 12 + (size_t)r2 * 4; }
 
 template <bool X3, int HC>
 __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_constant__ CUtensorMap map_hi,
@@ -182,20 +211,21 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
                                                    uint8_t* __restrict__ slots, unsigned* __restrict__ gflags) {
   using namespace tc;
   constexpr int NOPS = X3 ? 2 : 1;
-  constexpr int NP = 2 * HC, P = gram_pack(NP), KPB = gram_kpb(NP), KSB = KPB / P;
+  constexpr int NP = 2 * HC, KPB = gram_kpb(NP), KP = KPB / 2, HB = gram_hb(NP);
   extern __shared__ unsigned char smem_raw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sm = smem_align1024(smem_raw);
   GramHdr* hdr = reinterpret_cast<GramHdr*>(sm);
   uint8_t* stages = sm + 1024;
   const uint32_t op_bytes = a.box_bytes * KPB;           // one operand of an item
   const uint32_t stage_bytes = op_bytes * NOPS;          // [hi blocks][lo blocks]
+  const uint32_t stage0 = smem_u32(stages);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int64_t i0 = a.nitems * blockIdx.x / gridDim.x;
   const int64_t i1 = a.nitems * (blockIdx.x + 1) / gridDim.x;
   const int nit = (int)(i1 - i0);
   const int FB = a.flush;
-  const int nkb = (int)a.nkb, nsb = (int)a.nsb;
+  const int nkb = (int)a.nkb, nblk = (int)a.nblk;
 
   if (tid == 0) {
     for (int i = 0; i < a.nst; ++i) {
@@ -221,87 +251,129 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = hdr->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, hdr->tmem_base, 0);
   volatile int* abort_flag = &hdr->abort;
 
-  if (warp == kTmaWarp && lane == 0 && nit > 0) {
+  if (warp == kTmaWarp && nit > 0) {
     // ---------------- TMA producer
-    prefetch_tmap(&map_hi);
-    if (X3) prefetch_tmap(&map_lo);
+    const bool leader = elect_one();
+    if (leader) {
+      prefetch_tmap(&map_hi);
+      if (X3) prefetch_tmap(&map_lo);
+    }
     int issued = 0;
     const int skipped = a.stall0 ? 1 : 0;       // items at the head never issued (self-test)
-    Cursor cu;
-    cu.init(i0, nkb);
-    for (int i = 0; i < nit; ++i, cu.next(nkb, a.nst)) {
+    Cursor<KP> cu;
+    cu.init(i0, nit, nkb);
+    for (int i = 0; cu.more(); ++i, cu.next(nkb, a.nst)) {
       const int s = cu.s;
-      if (i >= a.nst && !mbar_wait(smem_u32(&hdr->empty[s]), cu.ph ^ 1, abort_flag, gflags)) break;
+      if (i >= a.nst && !mbar_wait_warp(smem_u32(&hdr->empty[s]), cu.ph ^ 1, abort_flag, gflags)) break;
       if (i < skipped) {
         issued = i + 1;
         continue;
       }
       const uint32_t fb = smem_u32(&hdr->full[s]);
-      mbar_arrive_expect_tx(fb, stage_bytes);
-      uint8_t* st = stages + (size_t)s * stage_bytes;
-      tma_load_4d(smem_u32(st), &map_hi, 0, 0, cu.f, cu.kp * KPB, fb);
-      if (X3) tma_load_4d(smem_u32(st + op_bytes), &map_lo, 0, 0, cu.f, cu.kp * KPB, fb);
+      const uint32_t st = stage0 + (uint32_t)s * stage_bytes;
+      if (leader) {
+        mbar_arrive_expect_tx(fb, stage_bytes);
+        tma_load_4d(st, &map_hi, 0, 0, cu.f, cu.kp * 2, fb);
+        if (X3) tma_load_4d(st + op_bytes, &map_lo, 0, 0, cu.f, cu.kp * 2, fb);
+      }
+      __syncwarp();
       issued = i + 1;
     }
     // copies still in flight must land before the CTA can exit
     for (int i = max(skipped, issued - a.nst); i < issued; ++i)
       mbar_drain(smem_u32(&hdr->full[i % a.nst]), (i / a.nst) & 1, gflags);
-  } else if (warp == kMmaWarp && lane == 0 && nit > 0) {
+  } else if (warp == kMmaWarp && nit > 0) {
     // ---------------- MMA issuer
-    const uint32_t idesc = idesc_bf16(128, P * NP, 0, 0);
-    GroupWalk gw;
-    Cursor cu;
-    cu.init(i0, nkb);
+    const uint32_t idesc = idesc_bf16(128, NP, 0, 0);
+    const bool leader = elect_one();
+    GroupWalk<HB> gw;
+    Cursor<KP> cu;
+    cu.init(i0, nit, nkb);
     bool ok = true;
-    for (int i = 0; i < nit && ok; ++i, cu.next(nkb, a.nst)) {
+    for (; cu.more() && ok; cu.next(nkb, a.nst)) {
       const int f = cu.f, kp = cu.kp;
       const int s = cu.s;
-      if (!mbar_wait(smem_u32(&hdr->full[s]), cu.ph, abort_flag, gflags)) break;
+      if (!mbar_wait_warp(smem_u32(&hdr->full[s]), cu.ph, abort_flag, gflags)) break;
       tc_fence_after();
-      const uint32_t st = smem_u32(stages + (size_t)s * stage_bytes);
-      // packs past the chunk's last one hold no data (blocks past the chunk's
-      // last one read as zeros)
-      const int nvalid = min(KSB, nsb - kp * KSB);
-      const bool item_last = i + 1 == nit || cu.last_of_f(nkb);
-      for (int j = 0; j < nvalid; ++j) {
-        const bool gstart = gw.step(f, FB, a.nacc);
-        const bool sstart = gw.sstart;              // only on an item's first block
-        const int g = gw.g, acc = gw.acc, sg = gw.seg, a2b = sg & 1;
-        const bool gend = (item_last && j + 1 == nvalid) || gw.in_group == FB;
-        // the buffer's previous run (use (g / nacc) - 1) must have been drained
-        if (gstart && g >= a.nacc &&
-            !mbar_wait(smem_u32(&hdr->accempty[acc]), gw.accph ^ 1, abort_flag, gflags)) {
-          ok = false;
+      const uint32_t st = stage0 + (uint32_t)s * stage_bytes;
+      // a block past the chunk's points (odd block count) holds no data of this chunk
+      const int nvalid = min(2 * cu.n, nblk - kp * 2);
+      const bool item_last = cu.seg_end(nkb);
+      if (HB == KPB && FB == 1) {
+        // a run per block and a group per item (no group spans two): the plain loop
+        gw.item(f, a.nacc);
+        const int acc = gw.acc, a2b = gw.seg & 1;
+        if (gw.g >= a.nacc && !mbar_wait_warp(smem_u32(&hdr->accempty[acc]), gw.accph ^ 1, abort_flag, gflags)) break;
+        if (X3 && gw.sstart && gw.seg >= 2 &&
+            !mbar_wait_warp(smem_u32(&hdr->a2empty[a2b]), ((gw.seg >> 1) - 1) & 1, abort_flag, gflags))
           break;
-        }
-        if (X3 && sstart && sg >= 2 &&
-            !mbar_wait(smem_u32(&hdr->a2empty[a2b]), ((sg >> 1) - 1) & 1, abort_flag, gflags)) {
-          ok = false;
-          break;
-        }
         tc_fence_after();
-        const uint32_t d1 = tmem + (uint32_t)(acc * P * NP);
-        const uint32_t d2 = tmem + (uint32_t)((a.nacc + a2b) * P * NP);
-        const uint32_t hi = st + (uint32_t)(j * P) * a.box_bytes;
-        const uint32_t lo = hi + op_bytes;
+        const uint32_t d2 = tmem + (uint32_t)((a.nacc * HB + a2b) * NP);
+        if (leader) {
+          uint32_t d1 = tmem + (uint32_t)(acc * HB * NP), c2 = gw.sstart ? 0u : 1u;
+          uint64_t dh = sdesc_sw128(st, 16, 1024), dl = sdesc_sw128(st + op_bytes, 16, 1024);
+          for (int j = 0; j < nvalid; ++j) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint64_t dh = sdesc_sw128(hi + k * 32, 16, 1024);
-          mma_bf16(d1, dh, dh, idesc, (gstart && k == 0) ? 0u : 1u);                // A1 (+)= hi hi^T
-          if (X3) {
-            const uint64_t dl = sdesc_sw128(lo + k * 32, 16, 1024);
-            mma_bf16(d2, dh, dl, idesc, (sstart && j == 0 && k == 0) ? 0u : 1u);   // A2 (+)= hi lo^T
+            for (int k = 0; k < 4; ++k) {
+              mma_bf16(d1, dh + 2 * k, dh + 2 * k, idesc, k == 0 ? 0u : 1u);
+              if (X3) {
+                mma_bf16(d2, dh + 2 * k, dl + 2 * k, idesc, c2);
+                c2 = 1u;
+              }
+            }
+            d1 += NP;
+            dh += NP * 128 / 16;
+            dl += NP * 128 / 16;
           }
+          mma_commit(smem_u32(&hdr->accfull[acc]));
         }
-        if (gend) mma_commit(smem_u32(&hdr->accfull[acc]));
+        __syncwarp();
+      } else {
+        for (int j = 0; j < nvalid; ++j) {
+          const bool gstart = gw.step(f, FB, a.nacc);
+          const bool sstart = gw.sstart;              // only on an item's first block
+          const int g = gw.g, acc = gw.acc, sg = gw.seg, a2b = sg & 1;
+          const bool gend = gw.ends(item_last && j + 1 == nvalid, FB);
+          // the buffer's previous group (use (g / nacc) - 1) must have been drained
+          if (gstart && g >= a.nacc &&
+              !mbar_wait_warp(smem_u32(&hdr->accempty[acc]), gw.accph ^ 1, abort_flag, gflags)) {
+            ok = false;
+            break;
+          }
+          if (X3 && sstart && sg >= 2 &&
+              !mbar_wait_warp(smem_u32(&hdr->a2empty[a2b]), ((sg >> 1) - 1) & 1, abort_flag, gflags)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t d1 = tmem + (uint32_t)((acc * HB + gw.run) * NP);
+          const uint32_t d2 = tmem + (uint32_t)((a.nacc * HB + a2b) * NP);
+          const uint32_t hi = st + (uint32_t)j * a.box_bytes;
+          const uint32_t lo = hi + op_bytes;
+          if (leader) {
+            const uint64_t dh0 = sdesc_sw128(hi, 16, 1024), dl0 = sdesc_sw128(lo, 16, 1024);
+            const uint32_t c1 = gw.rstart ? 0u : 1u, c2 = (sstart && j == 0) ? 0u : 1u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {            // K steps of 32 bytes
+              mma_bf16(d1, dh0 + 2 * k, dh0 + 2 * k, idesc, k == 0 ? c1 : 1u);             // A1 (+)= hi hi^T
+              if (X3) mma_bf16(d2, dh0 + 2 * k, dl0 + 2 * k, idesc, k == 0 ? c2 : 1u);     // A2 (+)= hi lo^T
+            }
+            if (gend) mma_commit(smem_u32(&hdr->accfull[acc]));
+          }
+          __syncwarp();
+        }
       }
-      if (ok) mma_commit(smem_u32(&hdr->empty[s]));
+      if (ok && leader) mma_commit(smem_u32(&hdr->empty[s]));
+      __syncwarp();
     }
-    mma_commit(smem_u32(&hdr->drain));
-    mbar_drain(smem_u32(&hdr->drain), 0, gflags);
+    if (leader) {
+      mma_commit(smem_u32(&hdr->drain));
+      mbar_drain(smem_u32(&hdr->drain), 0, gflags);
+    }
+    __syncwarp();
   } else if (X3 && warp >= kDiagWarp0 && nit > 0) {
     // ---------------- lo-square diagonal of every lo block.  Eight threads
     // share a row (one 16-byte chunk each, so a warp reads 512 contiguous
@@ -312,39 +384,42 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
     const int t = tid - kDiagWarp0 * 32;
     const int rsub = t >> 3, chunk = t & 7;
     constexpr int kRowsPer = NP / 8;                  // rows rsub + 8 j < NP
+    const uint8_t* const lo0 = stages + op_bytes + rsub * 128 + chunk * 16;
     float q[kRowsPer];
 #pragma unroll
     for (int j = 0; j < kRowsPer; ++j) q[j] = 0.f;
-    Cursor cu;
-    cu.init(i0, nkb);
-    for (int i = 0; i < nit; ++i, cu.next(nkb, a.nst)) {
+    Cursor<KP> cu;
+    cu.init(i0, nit, nkb);
+    for (; cu.more(); cu.next(nkb, a.nst)) {
       const int f = cu.f, kp = cu.kp;
-      const bool send = i + 1 == nit || cu.last_of_f(nkb);
+      const bool send = cu.seg_end(nkb);
       const int s = cu.s;
       if (!mbar_wait(smem_u32(&hdr->full[s]), cu.ph, abort_flag, gflags)) break;
-      const int nvalid = min(KSB, nsb - kp * KSB) * P;
-      for (int b = 0; b < nvalid; ++b) {
-        const uint8_t* lo = stages + (size_t)s * stage_bytes + op_bytes + (size_t)b * a.box_bytes;
+      const int nvalid = min(2 * cu.n, nblk - kp * 2);
+      // (rows past r2 are zeros in the stage; shared-memory loads in batches: this
+      // role must not hold the stages back)
+      const uint8_t* lo = lo0 + (size_t)s * stage_bytes;
+#pragma unroll 2
+      for (int b = 0; b < nvalid; ++b, lo += NP * 128) {
+        uint4 w4[kRowsPer];
+#pragma unroll
+        for (int j = 0; j < kRowsPer; ++j) w4[j] = *reinterpret_cast<const uint4*>(lo + j * 1024);
 #pragma unroll
         for (int j = 0; j < kRowsPer; ++j) {
-          const int r = rsub + 8 * j;
-          if (r < a.r2) {
-            const uint4 w4 = *reinterpret_cast<const uint4*>(lo + (size_t)r * 128 + chunk * 16);
-            const uint32_t ws[4] = {w4.x, w4.y, w4.z, w4.w};
-            float acc = 0.f;
+          const uint32_t ws[4] = {w4[j].x, w4[j].y, w4[j].z, w4[j].w};
+          float acc = 0.f;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float la = __uint_as_float(ws[e] << 16), lb = __uint_as_float(ws[e] & 0xFFFF0000u);
-              acc = fmaf(la, la, acc);
-              acc = fmaf(lb, lb, acc);
-            }
-            q[j] += acc;
+          for (int e = 0; e < 4; ++e) {
+            const float la = __uint_as_float(ws[e] << 16), lb = __uint_as_float(ws[e] & 0xFFFF0000u);
+            acc = fmaf(la, la, acc);
+            acc = fmaf(lb, lb, acc);
           }
+          q[j] += acc;
         }
       }
       mbar_arrive(smem_u32(&hdr->empty[s]));
       if (send) {
-        float* dg = reinterpret_cast<float*>(slots + ((size_t)blockIdx.x + (size_t)f) * P * gram_slot_bytes(a.r2) +
+        float* dg = reinterpret_cast<float*>(slots + ((size_t)blockIdx.x + (size_t)f) * gram_slot_bytes(a.r2) +
                                              (size_t)a.r2 * a.r2 * 12);
 #pragma unroll
         for (int j = 0; j < kRowsPer; ++j) {
@@ -359,44 +434,40 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       }
     }
   } else if (warp < kEpiWarps) {
-    // ---------------- epilogue: TMEM -> registers -> slots.  Lane (quad, lane)
-    // holds row 32 quad + lane of D: row lr of diagonal block sub.  Warp (quad,
-    // half) drains the HC columns of its half of that block; where the quad
-    // spans two diagonal blocks (they change at lane 16: NP is a multiple of
-    // 16) both blocks' columns are read and each lane keeps its own.  Of A1
-    // (symmetric) only the 8-column chunks that reach the upper triangle (some
-    // row of the warp <= some column of the chunk) are read and summed.
+    // ---------------- epilogue: TMEM -> registers -> slots.  Warp (quad,
+    // half) drains rows quad*32 .. +31 and the HC columns of its half; of A1
+    // (symmetric) only the 8-column chunks that reach the upper triangle
+    // (some row of the quad <= some column of the chunk) are read and summed.
     constexpr int CH = HC / 8;
-    constexpr bool kTwo = P > 1 && NP % 32 != 0;  // some quad spans two diagonal blocks
     const int quad = warp & 3, half = warp >> 2;
-    const int sub_lo = quad * 32 / NP, sub_hi = (quad * 32 + 16) / NP;
-    const bool two = kTwo && sub_hi != sub_lo && sub_hi < P;
-    const bool upper = two && lane >= 16;
-    const int sub = upper ? sub_hi : sub_lo;
-    const int row = quad * 32 + lane - sub * NP;  // row of the lane's diagonal block
-    const int rmin = two ? 0 : quad * 32 - sub_lo * NP;
+    const int row = quad * 32 + lane;
     const int col0 = half * HC;
-    const bool active = sub_lo < P && (two || rmin < a.r2);   // this lane quadrant holds rows of D
+    const bool active = quad * 32 < a.r2;         // this lane quadrant holds rows of D
     int nch = 0;                                  // chunks [CH - nch, CH) of this warp are upper-triangle ones
 #pragma unroll
-    for (int c = 0; c < CH; ++c) nch += (col0 + 8 * c + 7 >= rmin) ? 1 : 0;
+    for (int c = 0; c < CH; ++c) nch += (col0 + 8 * c + 7 >= quad * 32) ? 1 : 0;
     const int c_first = CH - nch;
     float s1[HC], c1[HC];
 #pragma unroll
     for (int j = 0; j < HC; ++j) { s1[j] = 0.f; c1[j] = 0.f; }
-    GroupWalk gw;
-    Cursor cu;
-    cu.init(i0, nkb);
+    GroupWalk<HB> gw;
+    Cursor<KP> cu;
+    cu.init(i0, nit, nkb);
     bool ok = true;
-    for (int i = 0; i < nit && ok; ++i, cu.next(nkb, a.nst)) {
+    for (; cu.more() && ok; cu.next(nkb, a.nst)) {
      const int f = cu.f;
-     const int nvalid = min(KSB, nsb - cu.kp * KSB);
-     const bool item_last = i + 1 == nit || cu.last_of_f(nkb);
-     for (int j = 0; j < nvalid; ++j) {
-      gw.step(f, FB, a.nacc);
+     const int nvalid = min(2 * cu.n, nblk - cu.kp * 2);
+     const bool item_last = cu.seg_end(nkb);
+     const bool plain = HB == KPB && FB == 1;         // the item is a group (see the MMA warp)
+     for (int j = plain ? nvalid - 1 : 0; j < nvalid; ++j) {
       const bool send = item_last && j + 1 == nvalid;
-      const bool gend = send || gw.in_group == FB;
-      if (!gend) continue;
+      if (plain) {
+        gw.item(f, a.nacc);
+        gw.run = nvalid - 1;
+      } else {
+        gw.step(f, FB, a.nacc);
+        if (!gw.ends(send, FB)) continue;
+      }
       const int acc = gw.acc, a2b = gw.seg & 1;
       // one decision per warp: the tcgen05.ld below must be executed by the whole warp
       const bool got = mbar_wait(smem_u32(&hdr->accfull[acc]), gw.accph, abort_flag, gflags);
@@ -406,42 +477,46 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       }
       tc_fence_after();
       if (active && nch > 0) {
-        // this warp's A1 chunks in one batch of loads and one wait
-        const uint32_t t1 =
-            tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * P * NP + sub_lo * NP) + (uint32_t)col0;
-        float v[HC];
+        // this warp's A1 chunks, LB runs in one batch of loads and one wait
+        constexpr int LB = HC * HB <= 64 ? HB : HC * 2 <= 64 && HB > 1 ? 2 : 1;
+        const uint32_t t1 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * HB * NP) + (uint32_t)col0;
 #pragma unroll
-        for (int c = 0; c < CH; ++c)
-          if (c >= c_first) tmem_ld8(t1 + (uint32_t)(c * 8), v + c * 8);
-        if (kTwo && two) {
-          float w[HC];
+        for (int r0 = 0; r0 < HB; r0 += LB) {
+          if (r0 > gw.run) break;
+          float v[LB][HC];
 #pragma unroll
-          for (int c = 0; c < CH; ++c)
-            if (c >= c_first) tmem_ld8(t1 + (uint32_t)(NP + c * 8), w + c * 8);
+          for (int r = 0; r < LB; ++r)
+            if (r0 + r <= gw.run) {
+#pragma unroll
+              for (int c = 0; c < CH; ++c)
+                if (c >= c_first) tmem_ld8(t1 + (uint32_t)((r0 + r) * NP + c * 8), v[r] + c * 8);
+            }
           tmem_wait_ld();
-#pragma unroll
-          for (int c = 0; c < HC; ++c) v[c] = upper ? w[c] : v[c];
-        } else {
-          tmem_wait_ld();
-        }
-        tc_fence_before();
-        mbar_arrive(smem_u32(&hdr->accempty[acc]));
-#pragma unroll
-        for (int c = 0; c < CH; ++c)
-          if (c >= c_first) {
-#pragma unroll
-            for (int e = 0; e < 8; e += 2)
-              kahan_add2(s1[c * 8 + e], s1[c * 8 + e + 1], c1[c * 8 + e], c1[c * 8 + e + 1], v[c * 8 + e],
-                         v[c * 8 + e + 1]);
+          if (r0 + LB > gw.run) {                  // the group's last batch: the buffer is free
+            tc_fence_before();
+            mbar_arrive(smem_u32(&hdr->accempty[acc]));
           }
+#pragma unroll
+          for (int r = 0; r < LB; ++r)
+            if (r0 + r <= gw.run) {
+#pragma unroll
+              for (int c = 0; c < CH; ++c)
+                if (c >= c_first) {
+#pragma unroll
+                  for (int e = 0; e < 8; e += 2)
+                    kahan_add2(s1[c * 8 + e], s1[c * 8 + e + 1], c1[c * 8 + e], c1[c * 8 + e + 1], v[r][c * 8 + e],
+                               v[r][c * 8 + e + 1]);
+                }
+            }
+        }
       } else {
         tc_fence_before();
         mbar_arrive(smem_u32(&hdr->accempty[acc]));
       }
       if (!send) continue;
       // the CTA's run of frequency f ends: its sums go to slot (cta + f)
-      uint8_t* slot = slots + (((size_t)blockIdx.x + (size_t)f) * P + sub) * gram_slot_bytes(a.r2);
-      const bool wr = row < a.r2 && sub < P;
+      uint8_t* slot = slots + ((size_t)blockIdx.x + (size_t)f) * gram_slot_bytes(a.r2);
+      const bool wr = row < a.r2;
       if (active) {
         float2* d1 = reinterpret_cast<float2*>(slot) + (size_t)row * a.r2 + col0;
 #pragma unroll
@@ -454,21 +529,12 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
       if (X3) {
         if (active) {
           // the segment's A2 (its MMAs completed with the last group's), not symmetric: all of it
-          const uint32_t t2 = tmem + ((uint32_t)(quad * 32) << 16) +
-                              (uint32_t)((a.nacc + a2b) * P * NP + sub_lo * NP) + (uint32_t)col0;
+          const uint32_t t2 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((a.nacc * HB + a2b) * NP) +
+                              (uint32_t)col0;
           float v[HC];
 #pragma unroll
           for (int c = 0; c < CH; ++c) tmem_ld8(t2 + (uint32_t)(c * 8), v + c * 8);
-          if (kTwo && two) {
-            float w[HC];
-#pragma unroll
-            for (int c = 0; c < CH; ++c) tmem_ld8(t2 + (uint32_t)(NP + c * 8), w + c * 8);
-            tmem_wait_ld();
-#pragma unroll
-            for (int c = 0; c < HC; ++c) v[c] = upper ? w[c] : v[c];
-          } else {
-            tmem_wait_ld();
-          }
+          tmem_wait_ld();
           tc_fence_before();
           mbar_arrive(smem_u32(&hdr->a2empty[a2b]));
           float* d2 = reinterpret_cast<float*>(slot + (size_t)a.r2 * a.r2 * 8) + (size_t)row * a.r2 + col0;
@@ -494,11 +560,11 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
 // CTA c's item range is [floor(c W / G), floor((c+1) W / G)); the CTA holding item i.
 __device__ __forceinline__ int64_t cta_of_item(int64_t i, int64_t W, int64_t G) { return ((i + 1) * G - 1) / W; }
 
-// acc[f] (+)= sum over the CTAs c that covered frequency f of the pack
-// sub-slots of slot (c + f), in CTA and sub-slot order, of D = A1 + A2 + A2^T +
-// diag(lo lo^T) (A1 as a compensated (sum, carry) pair, read from its upper triangle).
-__global__ void k_gram_tc_collect(const uint8_t* __restrict__ slots, int r2, int pack, int64_t nkb, int64_t G,
-                                  int x3, int first, double* __restrict__ acc) {
+// acc[f] (+)= sum over the CTAs c that covered frequency f of slot (c + f), in
+// CTA order, of D = A1 + A2 + A2^T + diag(lo lo^T) (A1 as a compensated (sum, carry)
+// pair, read from its upper triangle).
+__global__ void k_gram_tc_collect(const uint8_t* __restrict__ slots, int r2, int64_t nkb, int64_t G, int x3,
+                                  int first, double* __restrict__ acc) {
   const int f = blockIdx.x;
   const int64_t W = (int64_t)gridDim.x * nkb;
   const int64_t c0 = cta_of_item((int64_t)f * nkb, W, G);
@@ -506,28 +572,25 @@ __global__ void k_gram_tc_collect(const uint8_t* __restrict__ slots, int r2, int
   double* dst = acc + (int64_t)f * r2 * r2;
   const size_t sb = gram_slot_bytes(r2);
   // one entry (i <= j) of the symmetric D per thread: the conversions and sums
-  // in FP64 bound this kernel
+  // in FP64 bound this kernel (nf = 129, 31 rows: 13.8 us with 256 threads per
+  // frequency over all entries)
   const int t = blockIdx.y * blockDim.x + threadIdx.x;
   if (t < r2 * (r2 + 1) / 2) {
     int j = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
     while (j * (j + 1) / 2 > t) --j;
     while ((j + 1) * (j + 2) / 2 <= t) ++j;
     const int i = t - j * (j + 1) / 2;
-    const int e = i * r2 + j;
-    double v = 0.0;
-    const int et = j * r2 + i;
+    const int e = i * r2 + j, et = j * r2 + i;
     const size_t o2 = (size_t)r2 * r2 * 8;
-    const uint8_t* slot = slots + (size_t)(c0 + f) * pack * sb;
-    for (int c = 0; c <= (int)(c1 - c0); ++c) {
-      if (x3 && i == j) v += (double)reinterpret_cast<const float*>(slot + o2 + (size_t)r2 * r2 * 4)[i];
-#pragma unroll 8
-      for (int q = 0; q < pack; ++q, slot += sb) {
-        const float2 sc = reinterpret_cast<const float2*>(slot)[e];   // A1: upper triangle only
-        v += (double)sc.x + (double)sc.y;
-        if (x3) {
-          const float* a2 = reinterpret_cast<const float*>(slot + o2);
-          v += (double)a2[e] + (double)a2[et];
-        }
+    double v = 0.0;
+    const uint8_t* slot = slots + (size_t)(c0 + f) * sb;
+    for (int c = 0; c <= (int)(c1 - c0); ++c, slot += sb) {
+      const float2 sc = reinterpret_cast<const float2*>(slot)[e];   // A1: upper triangle only
+      v += (double)sc.x + (double)sc.y;
+      if (x3) {
+        const float* a2 = reinterpret_cast<const float*>(slot + o2);
+        v += (double)a2[e] + (double)a2[et];
+        if (i == j) v += (double)reinterpret_cast<const float*>(slot + o2 + (size_t)r2 * r2 * 4)[i];
       }
     }
     v = first ? v : dst[e] + v;
@@ -580,7 +643,7 @@ size_t gram_tc_smem_stages(const spod_plan_s& p, int nst) {
   const int nops = p.desc.precision == SPOD_PREC_BF16X3 ? 2 : 1;
   const size_t np = (size_t)((2 * p.nb + 15) / 16 * 16);
   // + the rows an M = 128 A operand reads past the last stage's last block
-  return 1024 + 1024 + (size_t)nst * nops * gram_kpb((int)np) * np * 128 + (128 - gram_pack((int)np) * np) * 128;
+  return 1024 + 1024 + (size_t)nst * nops * gram_kpb((int)np) * np * 128 + (128 - np) * 128;
 }
 
 template <bool X3, int HC>
@@ -615,11 +678,11 @@ cudaError_t launch_gram_tc_x(const spod_plan_s& p, const CUtensorMap& mh, const 
 // Shared memory of the smallest (2-stage) configuration; launches use up to 8 stages.
 size_t gram_tc_smem_bytes(const spod_plan_s& p) { return gram_tc_smem_stages(p, 2); }
 
-// Slots of the persistent kernel, (max CTAs + nf - 1) x pack x gram_slot_bytes(qrows)
+// Slots of the persistent kernel, (max CTAs + nf - 1) x gram_slot_bytes(qrows)
 // (counted in doubles), and the per-frequency FP64 accumulator of D over
 // chunks, nf x qrows^2 (qrows = 2 nb, + 1 with the folded mean's rho row).
 size_t gram_tc_slot_doubles(const spod_plan_s& p, int max_ctas) {
-  return (size_t)(max_ctas + p.nf - 1) * gram_pack((2 * p.nb + 15) / 16 * 16) * gram_slot_bytes(p.qrows) / 8;
+  return ((size_t)(max_ctas + p.nf - 1) * gram_slot_bytes(p.qrows) + 7) / 8;
 }
 size_t gram_tc_acc_doubles(const spod_plan_s& p) { return (size_t)p.nf * p.qrows * p.qrows; }
 
@@ -638,14 +701,13 @@ cudaError_t launch_gram_tc_chunk(const spod_plan_s& p, int64_t mcount, bool firs
   a.flush = p.gram_flush > 0 ? p.gram_flush : 1;
   a.box_bytes = (uint32_t)a.np * 128u;
   // A1 buffers: as many as the 512 tensor-memory columns hold beside the two
-  // A2 buffers (np = 80 for nb = 38: four; packed blocks: two or three of P
-  // blocks each), so that short A1 runs are drained while the next ones accumulate
-  const int pack = gram_pack(a.np), kpb = gram_kpb(a.np), ncol = pack * a.np;
-  a.nacc = std::max(2, std::min(kMaxAcc, ((int)kTmemCols - 2 * ncol) / ncol));
+  // A2 buffers (np = 80 for nb = 38: four), so that short A1 runs are drained
+  // while the next ones accumulate
+  const int kpb = gram_kpb(a.np);
+  a.nacc = std::max(2, std::min(kMaxAcc, ((int)kTmemCols - 2 * a.np) / (gram_hb(a.np) * a.np)));
   a.stall0 = p.wait_selftest ? 1 : 0;
-  const int64_t nblk = (mcount + 63) / 64;
-  a.nsb = (nblk + pack - 1) / pack;
-  a.nkb = (nblk + kpb - 1) / kpb;
+  a.nblk = (mcount + 63) / 64;
+  a.nkb = (a.nblk + 1) / 2;
   a.nitems = a.nkb * p.nf;
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p.device);
@@ -653,15 +715,15 @@ cudaError_t launch_gram_tc_chunk(const spod_plan_s& p, int64_t mcount, bool firs
   while (a.nst > 2 && gram_tc_smem_stages(p, a.nst) > (size_t)optin) --a.nst;
   const size_t smem = gram_tc_smem_stages(p, a.nst);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(gram_tc_ctas(p), a.nitems));
-  // maps whose last block is the chunk's: what a box reads past it is zero
+  // maps whose last block is the chunk's (a box may reach past it)
   CUtensorMap mh, ml;
-  if (!make_qhat_map(p, p.d_qhat, kpb, nblk, &mh) || !make_qhat_map(p, p.d_qlo ? p.d_qlo : p.d_qhat, kpb, nblk, &ml))
+  if (!make_qhat_map(p, p.d_qhat, kpb, a.nblk, &mh) || !make_qhat_map(p, p.d_qlo ? p.d_qlo : p.d_qhat, kpb, a.nblk, &ml))
     return cudaErrorUnknown;
   cudaError_t e = p.desc.precision == SPOD_PREC_BF16X3 ? launch_gram_tc_x<true>(p, mh, ml, a, grid, smem, s)
                                                         : launch_gram_tc_x<false>(p, mh, ml, a, grid, smem, s);
   if (e != cudaSuccess) return e;
   k_gram_tc_collect<<<dim3((unsigned)p.nf, (unsigned)((a.r2 * (a.r2 + 1) / 2 + 127) / 128)), 128, 0, s>>>(
-      reinterpret_cast<const uint8_t*>(p.d_gslot), a.r2, pack, a.nkb, grid,
+      reinterpret_cast<const uint8_t*>(p.d_gslot), a.r2, a.nkb, grid,
                                          p.desc.precision == SPOD_PREC_BF16X3 ? 1 : 0, first ? 1 : 0, p.d_gacc);
   return cudaGetLastError();
 }

@@ -25,10 +25,11 @@
 //
 // What bounds it: HBM (Qhat read, Phi written), as long as enough bytes are in
 // flight and no tile waits for a hand-over.  Hence items of about 32 KB whatever
-// nb is, one hand-over per item, and sixteen draining warps: 361 x 720 x 2
-// points, 361 bins, nb = 7, three modes 10.7 -> 2.6 ms (6.0 TB/s); nb = 21, 193
-// bins, five modes 6.1 -> 3.6 ms; 512 x 256 x 3 points, nb = 38, five modes
-// 6.5 -> 5.2 ms (6.7 TB/s), 38 modes of a quarter of it 2.62 -> 2.46 ms.
+// nb is, one hand-over per item, sixteen draining warps, and issuing warps that run
+// as whole warps (elect_one): 361 x 720 x 2 points, 361 bins, nb = 7, three modes
+// 10.7 -> 2.4 ms (6.4 TB/s); nb = 21, 193 bins, five modes 6.1 -> 3.3 ms; BF16, nb = 33,
+// 129 bins, five modes 4.2 -> 1.7 ms; 512 x 256 x 3 points, nb = 38, five modes
+// 6.5 -> 5.1 ms (6.9 TB/s).
 #include <algorithm>
 
 #include "tc_common.cuh"
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
   using namespace tc;
   constexpr int NOPS = X3 ? 2 : 1;
   extern __shared__ unsigned char smem_raw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sm = smem_align1024(smem_raw);
   ModesHdr* hdr = reinterpret_cast<ModesHdr*>(sm);
   uint8_t* Bhi = sm + 1024;
   uint8_t* Blo = Bhi + a.img_bytes;
@@ -174,8 +175,9 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
   const uint32_t op_bytes = tile_bytes * a.tiles;
   const uint32_t stage_bytes = op_bytes * NOPS;           // [hi tiles][lo tiles]
   uint8_t* stages = Bhi + NOPS * a.img_bytes;
+  const uint32_t stage0 = smem_u32(stages);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int64_t i0 = a.nitems * blockIdx.x / gridDim.x;
   const int64_t i1 = a.nitems * (blockIdx.x + 1) / gridDim.x;
   const int nit = (int)(i1 - i0);
@@ -203,13 +205,16 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = hdr->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, hdr->tmem_base, 0);
   volatile int* abort_flag = &hdr->abort;
 
-  if (warp == kTmaWarp && lane == 0 && nit > 0) {
+  if (warp == kTmaWarp && nit > 0) {
     // ---------------- TMA producer (+ B image at each frequency change)
-    prefetch_tmap(&map_hi);
-    if (X3) prefetch_tmap(&map_lo);
+    const bool leader = elect_one();
+    if (leader) {
+      prefetch_tmap(&map_hi);
+      if (X3) prefetch_tmap(&map_lo);
+    }
     int issued = 0, seg = 0, segs_loaded = 0;
     int fcur = -1;
     Cursor cu;
@@ -218,35 +223,42 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
       const int f = cu.f, tp = cu.tp;
       if (f != fcur) {
         // the MMAs of the previous frequency must be done with B before it is replaced
-        if (seg >= 1 && !mbar_wait(smem_u32(&hdr->bempty), (seg - 1) & 1, abort_flag, gflags)) break;
+        if (seg >= 1 && !mbar_wait_warp(smem_u32(&hdr->bempty), (seg - 1) & 1, abort_flag, gflags)) break;
         const uint32_t bb = smem_u32(&hdr->bfull);
-        mbar_arrive_expect_tx(bb, a.img_bytes * NOPS);
         const uint8_t* src = img + (size_t)f * a.img_bytes * NOPS;
-        bulk_load(smem_u32(Bhi), src, a.img_bytes, bb);
-        if (X3) bulk_load(smem_u32(Blo), src + a.img_bytes, a.img_bytes, bb);
+        if (leader) {
+          mbar_arrive_expect_tx(bb, a.img_bytes * NOPS);
+          bulk_load(smem_u32(Bhi), src, a.img_bytes, bb);
+          if (X3) bulk_load(smem_u32(Blo), src + a.img_bytes, a.img_bytes, bb);
+        }
+        __syncwarp();
         segs_loaded = seg + 1;
         fcur = f;
         ++seg;
       }
       const int s = cu.s;
-      if (i >= a.nst && !mbar_wait(smem_u32(&hdr->empty[s]), cu.ph ^ 1, abort_flag, gflags)) break;
+      if (i >= a.nst && !mbar_wait_warp(smem_u32(&hdr->empty[s]), cu.ph ^ 1, abort_flag, gflags)) break;
       const uint32_t fb = smem_u32(&hdr->full[s]);
-      mbar_arrive_expect_tx(fb, stage_bytes);
-      uint8_t* st = stages + (size_t)s * stage_bytes;
+      const uint32_t st = stage0 + (uint32_t)s * stage_bytes;
       const int kb = 2 * (tp * T + (int)a.qtile0);
       // one copy per operand: the item's 64-point blocks side by side
-      tma_load_4d(smem_u32(st), &map_hi, 0, 0, f, kb, fb);
-      if (X3) tma_load_4d(smem_u32(st + op_bytes), &map_lo, 0, 0, f, kb, fb);
+      if (leader) {
+        mbar_arrive_expect_tx(fb, stage_bytes);
+        tma_load_4d(st, &map_hi, 0, 0, f, kb, fb);
+        if (X3) tma_load_4d(st + op_bytes, &map_lo, 0, 0, f, kb, fb);
+      }
+      __syncwarp();
       issued = i + 1;
     }
     // copies still in flight must land before the CTA can exit
     for (int i = max(0, issued - a.nst); i < issued; ++i)
       mbar_drain(smem_u32(&hdr->full[i % a.nst]), (i / a.nst) & 1, gflags);
     if (segs_loaded > 0) mbar_drain(smem_u32(&hdr->bfull), (segs_loaded - 1) & 1, gflags);
-  } else if (warp == kMmaWarp && lane == 0 && nit > 0) {
+  } else if (warp == kMmaWarp && nit > 0) {
     // ---------------- MMA issuer
     const uint32_t idesc = idesc_bf16(128, a.nn, 1, 0);      // A MN-major (points), B K-major
     const uint32_t bhi = smem_u32(Bhi), blo = smem_u32(Blo);
+    const bool leader = elect_one();
     const uint32_t katom_bytes = (uint32_t)a.nn * 128u;
     const int nk16 = a.np / 16;
     int seg = 0;
@@ -256,41 +268,47 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
     for (int i = 0; i < nit; ++i, cu.next(nitf, a.nst)) {
       const int f = cu.f;
       if (f != fcur) {
-        if (seg >= 1) mma_commit(smem_u32(&hdr->bempty));   // B of the previous frequency is released
-        if (!mbar_wait(smem_u32(&hdr->bfull), seg & 1, abort_flag, gflags)) break;
+        if (seg >= 1 && leader) mma_commit(smem_u32(&hdr->bempty));   // B of the previous frequency is released
+        if (!mbar_wait_warp(smem_u32(&hdr->bfull), seg & 1, abort_flag, gflags)) break;
         fcur = f;
         ++seg;
       }
       const int s = cu.s;
-      if (!mbar_wait(smem_u32(&hdr->full[s]), cu.ph, abort_flag, gflags)) break;
+      if (!mbar_wait_warp(smem_u32(&hdr->full[s]), cu.ph, abort_flag, gflags)) break;
       tc_fence_after();
-      const uint32_t st = smem_u32(stages + (size_t)s * stage_bytes);
+      const uint32_t st = stage0 + (uint32_t)s * stage_bytes;
       const int acc = i % kAcc;
-      if (i >= kAcc && !mbar_wait(smem_u32(&hdr->accempty[acc]), (i / kAcc - 1) & 1, abort_flag, gflags)) break;
+      if (i >= kAcc && !mbar_wait_warp(smem_u32(&hdr->accempty[acc]), (i / kAcc - 1) & 1, abort_flag, gflags)) break;
       tc_fence_after();
       const int nv = min(T, ntp - cu.tp * T);
-      for (int t = 0; t < nv; ++t) {
-        const uint32_t d = tmem + (uint32_t)(acc * 128 + t * a.nn);
-        const uint32_t ta = st + (uint32_t)t * tile_bytes;
-        for (int j = 0; j < nk16; ++j) {
+      if (leader) {
+        for (int t = 0; t < nv; ++t) {
+          const uint32_t d = tmem + (uint32_t)(acc * 128 + t * a.nn);
           // A: 16 K rows of both point boxes (MN atoms box_bytes apart); B: 16 K columns
-          const uint64_t da = sdesc_sw128(ta + (uint32_t)j * 2048u, a.box_bytes, 1024);
-          const uint32_t boff = (uint32_t)(j >> 2) * katom_bytes + (uint32_t)(j & 3) * 32u;
-          const uint64_t db = sdesc_sw128(bhi + boff, 16, 1024);
-          mma_bf16(d, da, db, idesc, j > 0 ? 1u : 0u);
-          if (X3) {
-            const uint64_t dal = sdesc_sw128(ta + op_bytes + (uint32_t)j * 2048u, a.box_bytes, 1024);
-            const uint64_t dbl = sdesc_sw128(blo + boff, 16, 1024);
-            mma_bf16(d, da, dbl, idesc, 1u);
-            mma_bf16(d, dal, db, idesc, 1u);
+          const uint64_t da0 = sdesc_sw128(st + (uint32_t)t * tile_bytes, a.box_bytes, 1024);
+          const uint64_t dl0 = sdesc_sw128(st + (uint32_t)t * tile_bytes + op_bytes, a.box_bytes, 1024);
+          for (int j = 0; j < nk16; ++j) {
+            const uint64_t da = da0 + (uint64_t)(j * 128), dal = dl0 + (uint64_t)(j * 128);      // 2048 bytes
+            const uint32_t boff = (uint32_t)(j >> 2) * katom_bytes + (uint32_t)(j & 3) * 32u;
+            const uint64_t db = sdesc_sw128(bhi + boff, 16, 1024);
+            mma_bf16(d, da, db, idesc, j > 0 ? 1u : 0u);
+            if (X3) {
+              const uint64_t dbl = sdesc_sw128(blo + boff, 16, 1024);
+              mma_bf16(d, da, dbl, idesc, 1u);
+              mma_bf16(d, dal, db, idesc, 1u);
+            }
           }
         }
+        mma_commit(smem_u32(&hdr->empty[s]));
+        mma_commit(smem_u32(&hdr->accfull[acc]));
       }
-      mma_commit(smem_u32(&hdr->empty[s]));
-      mma_commit(smem_u32(&hdr->accfull[acc]));
+      __syncwarp();
     }
-    mma_commit(smem_u32(&hdr->drain));
-    mbar_drain(smem_u32(&hdr->drain), 0, gflags);
+    if (leader) {
+      mma_commit(smem_u32(&hdr->drain));
+      mbar_drain(smem_u32(&hdr->drain), 0, gflags);
+    }
+    __syncwarp();
   } else if (warp < kEpiWarps) {
     // ---------------- epilogue: TMEM -> registers -> scaled complex stores.
     // Groups of four warps (one per lane quadrant) take the CTA's items in turn;
