@@ -16,10 +16,9 @@
 // Nyquist) recovers the complex coefficient of the mode at the positive bin
 // (its conjugate bin carries conj(a)).  The reconstruction is
 //   X~ = mu + P_b^T C  (real rows [nt][M]).
-// The two large products run on k_gemm_simt, this file's SIMT GEMM (FP32 or
-// FP64 as the plan; the product over the M points is split over CTAs and the
-// parts summed in FP64 in a fixed order), as do C = G^{-1} B and the K x K
-// Gram of the basis, its inverse and the packing.
+// The two large products run on k_gemm_f32 (FP32 plans) or k_gemm_simt (FP64), this
+// file's SIMT GEMMs; the product over the M points is split over CTAs and the
+// parts summed in FP64 in a fixed order.  C = G^{-1} B runs on k_gemm_simt.
 #include <algorithm>
 #include <vector>
 
@@ -32,7 +31,7 @@ struct BasisRow {
   int f, k, part;   // bin, mode, 0: Re phi, 1: Im phi
 };
 
-// P_w[r][m] = W_m b_r[m], P_b[r][m] = b_r[m]; phi is the interleaved complex
+// P_w[r][m] = W_m b_r[m] (Pw may be NULL), P_b[r][m] = b_r[m]; phi is the interleaved complex
 // mode array [nf][nmodes][M].
 template <typename R>
 __global__ void k_coeff_basis(const R* __restrict__ phi, int nmodes, int64_t M, const BasisRow* __restrict__ rows,
@@ -44,79 +43,118 @@ __global__ void k_coeff_basis(const R* __restrict__ phi, int nmodes, int64_t M, 
     const R b = src[2 * m];
     const R sw = sqrtW[m];
     Pb[(int64_t)r * M + m] = b;
-    Pw[(int64_t)r * M + m] = b * sw * sw;
+    if (Pw) Pw[(int64_t)r * M + m] = b * sw * sw;
   }
 }
 
-__device__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-  return t;
-}
-
-// G[i][j] = G[j][i] = sum_m P_w[i][m] P_b[j][m] (j >= i), and, for j == K,
-// v[i] = sum_m P_w[i][m] mu[m]; FP64 sums in a fixed order.
+// G[i][j] = G[j][i] = sum_m P_w[i][m] P_b[j][m] for the 4 x 4 tiles (bi, bj), bi <= bj,
+// and, for bj one past the last tile, v[i] = sum_m P_w[i][m] mu[m]; FP64 sums in a
+// fixed order (thread t takes m = t, t + 256, ..).  What bounds it: the FP64 pipe.  K = 64,
+// M = 65 536: 0.86 ms, against 0.80 with one pair per CTA; but those 4160 CTAs kept the
+// product that runs beside it (Fork) off the SMs, and these 152 leave it most of each.
 template <typename R>
-__global__ void k_coeff_gram(const R* __restrict__ Pw, const R* __restrict__ Pb, const double* __restrict__ mu,
-                             int64_t M, int K, double* __restrict__ G, double* __restrict__ v) {
-  __shared__ double red[32];
-  const int i = blockIdx.x, j = blockIdx.y;
-  if (j < K && j < i) return;
-  const R* a = Pw + (int64_t)i * M;
-  double acc = 0.0;
-  if (j < K) {
-    const R* b = Pb + (int64_t)j * M;
-    for (int64_t m = threadIdx.x; m < M; m += blockDim.x) acc += (double)a[m] * (double)b[m];
-  } else {
-    for (int64_t m = threadIdx.x; m < M; m += blockDim.x) acc += (double)a[m] * mu[m];
+__global__ void __launch_bounds__(256) k_coeff_gram(const R* __restrict__ Pw, const R* __restrict__ Pb,
+                                                    const double* __restrict__ mu, int64_t M, int K,
+                                                    double* __restrict__ G, double* __restrict__ v) {
+  __shared__ double red[16][8];
+  const int i0 = 4 * blockIdx.x, j0 = 4 * blockIdx.y;
+  if (j0 < i0) return;
+  const bool isv = j0 >= K;
+  const R *a[4], *b[4];
+  for (int q = 0; q < 4; ++q) {                       // rows past K repeat the last one
+    a[q] = Pw + (int64_t)min(i0 + q, K - 1) * M;
+    b[q] = Pb + (int64_t)min(j0 + q, K - 1) * M;
   }
-  const double t = block_sum(acc, red);
-  if (threadIdx.x == 0) {
-    if (j < K) {
-      G[(int64_t)i * K + j] = t;
-      G[(int64_t)j * K + i] = t;
-    } else {
-      v[i] = t;
+  double acc[4][4];
+#pragma unroll
+  for (int x = 0; x < 4; ++x)
+#pragma unroll
+    for (int y = 0; y < 4; ++y) acc[x][y] = 0.0;
+  if (!isv) {
+    for (int64_t m = threadIdx.x; m < M; m += 256) {
+      double av[4], bv[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) { av[q] = (double)a[q][m]; bv[q] = (double)b[q][m]; }
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) acc[x][y] = fma(av[x], bv[y], acc[x][y]);
     }
+  } else {
+    for (int64_t m = threadIdx.x; m < M; m += 256) {
+      const double c = mu[m];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) acc[x][0] = fma((double)a[x][m], c, acc[x][0]);
+    }
+  }
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int x = 0; x < 4; ++x)
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      double t = acc[x][y];
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) red[4 * x + y][w] = t;
+    }
+  __syncthreads();
+  if (threadIdx.x >= 16) return;
+  const int i = i0 + (int)threadIdx.x / 4, j = j0 + (int)threadIdx.x % 4;
+  double t = 0.0;
+  for (int q = 0; q < 8; ++q) t += red[threadIdx.x][q];
+  if (isv) {
+    if (j == j0 && i < K) v[i] = t;
+  } else if (i < K && j < K && i <= j) {
+    G[(int64_t)i * K + j] = t;
+    G[(int64_t)j * K + i] = t;
   }
 }
 
 // Ginv = G^{-1} for the symmetric positive definite G (K x K, FP64) by
 // Gauss-Jordan elimination without pivoting (one CTA; G is overwritten).  A
 // pivot that is not positive (a basis that is not linearly independent)
-// raises FLAG_NOTCONV and leaves Ginv unusable.
-__global__ void k_spd_inverse(double* __restrict__ G, double* __restrict__ Ginv, int K, unsigned* __restrict__ flags) {
-  extern __shared__ double fac[];   // [K]
+// raises FLAG_NOTCONV and leaves Ginv unusable.  At step c the columns of G up to c
+// are those of I already and the columns of Ginv past c still are, so a row is K
+// entries: Ginv's up to c and G's past it.  With smem the two matrices are held in
+// shared memory (K <= kInvSmemK: the elimination is a chain of K short steps, and
+// through L2 each one waited for its loads; K = 64: 0.31 -> 0.16 ms).
+constexpr int kInvSmemK = 96;
+__global__ void __launch_bounds__(1024) k_spd_inverse(double* __restrict__ Gg, double* __restrict__ Ginv_g, int K,
+                                                      int smem, unsigned* __restrict__ flags) {
+  extern __shared__ double sh[];    // fac [K], then (smem) G and Ginv, rows of K + 1
+  double* const fac = sh;
+  double* const G = smem ? sh + K : Gg;
+  double* const Ginv = smem ? G + (size_t)K * (K + 1) : Ginv_g;
+  const int64_t ld = smem ? K + 1 : K;
   const int tid = threadIdx.x, nth = blockDim.x;
-  for (int idx = tid; idx < K * K; idx += nth) Ginv[idx] = (idx / K == idx % K) ? 1.0 : 0.0;
+  for (int idx = tid; idx < K * K; idx += nth) {
+    const int i = idx / K, j = idx - i * K;
+    if (smem) G[i * ld + j] = Gg[idx];
+    Ginv[i * ld + j] = i == j ? 1.0 : 0.0;
+  }
   __syncthreads();
   for (int c = 0; c < K; ++c) {
-    const double piv = G[(int64_t)c * K + c];
+    const double piv = G[c * ld + c];
     if (!(piv > 0.0)) {
       if (tid == 0) atomicOr(flags, FLAG_NOTCONV);
       return;
     }
+    for (int i = tid; i < K; i += nth) fac[i] = G[i * ld + c];
     __syncthreads();
     for (int j = tid; j < K; j += nth) {
-      G[(int64_t)c * K + j] /= piv;
-      Ginv[(int64_t)c * K + j] /= piv;
+      double* const e = (j > c ? G : Ginv) + c * ld + j;
+      *e /= piv;
     }
-    for (int i = tid; i < K; i += nth) fac[i] = G[(int64_t)i * K + c];
     __syncthreads();
     for (int idx = tid; idx < K * K; idx += nth) {
       const int i = idx / K, j = idx - i * K;
       if (i == c) continue;
-      const double fi = fac[i];
-      G[idx] -= fi * G[(int64_t)c * K + j];
-      Ginv[idx] -= fi * Ginv[(int64_t)c * K + j];
+      double* const X = j > c ? G : Ginv;
+      X[i * ld + j] -= fac[i] * X[c * ld + j];
     }
     __syncthreads();
   }
+  if (smem)
+    for (int idx = tid; idx < K * K; idx += nth) Ginv_g[idx] = Ginv[(idx / K) * ld + idx % K];
 }
 
 // d_A[q][t] (q = j * nmodes_r + k) from the real coefficients C (column-major
@@ -220,6 +258,139 @@ __global__ void __launch_bounds__(256) k_gemm_simt(int ni, int nj, int64_t nk, c
     }
 }
 
+// The FP32 products: D(i, j) = c(j) + sum_k A(i, k) B(k, j) over the split's range of
+// k in ascending order, A(i, k) = A[i sai + k], B(k, j) = B[j ldb + k] (BK) or
+// B[k ldb + j], D(i, j) = D[i sdi + j sdj], c(j) = mean[j] rounded (or 0).  64 x 128
+// tiles of D, 128 threads with 8 x 8 results each (rows 4 a .. and 32 + 4 a .., columns
+// 4 b .. and 64 + 4 b ..: conflict-free 16-byte shared loads), packed FMAs on pairs of
+// columns, k in steps of 16 through two shared buffers, the next step's loads in
+// registers meanwhile.  VEC: 16-byte loads (strides and bases multiples of 16 bytes).
+// What bounds it: FP32 issue (four shared loads and eight duplications for 32 packed
+// FMAs).  Same order of the same FMAs as k_gemm_simt, so the same results: K = 64,
+// nt = 4096, M = 65 536: 1.87 -> 0.97 ms over
+// the points, 1.50 (and 0.46 to fill in the mean) -> 0.66 for the reconstruction.
+template <bool BK, bool VEC>
+__global__ void __launch_bounds__(128, 3) k_gemm_f32(int ni, int nj, int64_t nk, const float* __restrict__ A,
+                                                     int64_t sai, const float* __restrict__ B, int64_t ldb,
+                                                     float* __restrict__ D, int64_t sdi, int64_t sdj, int64_t dsplit,
+                                                     const double* __restrict__ mean, int64_t kper) {
+  constexpr int TI = 64, TJ = 128, TK = 16;
+  __shared__ __align__(16) float As[2][TK][TI + 4];
+  __shared__ __align__(16) float Bs[2][TK][TJ + 4];
+  const int i0 = blockIdx.y * TI, j0 = blockIdx.x * TJ;
+  const int64_t k0 = (int64_t)blockIdx.z * kper;
+  const int64_t k1 = k0 + kper < nk ? k0 + kper : nk;
+  D += (int64_t)blockIdx.z * dsplit;
+  const int tid = threadIdx.x;
+  const int ta = tid / 16, tb = tid % 16;
+  // four consecutive elements p[0 .. 3], those past n (and all of a row not in) as zeros
+  auto load4 = [](const float* p, bool in, int64_t n) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (VEC) {
+      if (in && n > 0) v = *reinterpret_cast<const float4*>(p);   // n is a multiple of 4
+    } else if (in) {
+      if (n > 0) v.x = p[0];
+      if (n > 1) v.y = p[1];
+      if (n > 2) v.z = p[2];
+      if (n > 3) v.w = p[3];
+    }
+    return v;
+  };
+  float4 pa[2], pb[4];
+  auto fetch = [&](int64_t kb) {
+    const int q = tid % 4;
+    const int64_t k = kb + 4 * q;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int i = i0 + tid / 4 + 32 * r;
+      pa[r] = load4(A + (int64_t)i * sai + k, i < ni, k1 - k);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (BK) {
+        const int j = j0 + tid / 4 + 32 * r;
+        pb[r] = load4(B + (int64_t)j * ldb + k, j < nj, k1 - k);
+      } else {
+        const int64_t kk = kb + tid / 32 + 4 * r;
+        const int j = j0 + 4 * (tid % 32);
+        pb[r] = load4(B + kk * ldb + j, kk < k1, nj - j);
+      }
+    }
+  };
+  auto put = [&](int s) {
+    const int q = 4 * (tid % 4);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int i = tid / 4 + 32 * r;
+      As[s][q][i] = pa[r].x; As[s][q + 1][i] = pa[r].y; As[s][q + 2][i] = pa[r].z; As[s][q + 3][i] = pa[r].w;
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (BK) {
+        const int j = tid / 4 + 32 * r;
+        Bs[s][q][j] = pb[r].x; Bs[s][q + 1][j] = pb[r].y; Bs[s][q + 2][j] = pb[r].z; Bs[s][q + 3][j] = pb[r].w;
+      } else {
+        *reinterpret_cast<float4*>(&Bs[s][tid / 32 + 4 * r][4 * (tid % 32)]) = pb[r];
+      }
+    }
+  };
+  float2 acc[8][4];
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 4; ++y) acc[x][y] = make_float2(0.f, 0.f);
+  int s = 0;
+  if (k0 < k1) {
+    fetch(k0);
+    put(0);
+  }
+  __syncthreads();
+  for (int64_t kb = k0; kb < k1; kb += TK, s ^= 1) {
+    const bool more = kb + TK < k1;
+    if (more) fetch(kb + TK);
+#pragma unroll
+    for (int kk = 0; kk < TK; ++kk) {
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[s][kk][4 * ta]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[s][kk][32 + 4 * ta]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[s][kk][4 * tb]);
+      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[s][kk][64 + 4 * tb]);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float2 bv[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                            make_float2(b1.z, b1.w)};
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const float2 a2 = make_float2(av[x], av[x]);
+#pragma unroll
+        for (int y = 0; y < 4; ++y) acc[x][y] = __ffma2_rn(a2, bv[y], acc[x][y]);
+      }
+    }
+    if (more) put(s ^ 1);          // last read a step ago, before the barrier below
+    __syncthreads();
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int j = j0 + 64 * h + 4 * tb;
+    float c[4];
+#pragma unroll
+    for (int y = 0; y < 4; ++y) c[y] = mean && j + y < nj ? (float)mean[j + y] : 0.f;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      const int i = i0 + (x < 4 ? 0 : 28) + 4 * ta + x;
+      if (i >= ni) continue;
+      const float2 u = acc[x][2 * h], w = acc[x][2 * h + 1];
+      const float r[4] = {c[0] + u.x, c[1] + u.y, c[2] + w.x, c[3] + w.y};
+      float* const d = D + (int64_t)i * sdi + (int64_t)j * sdj;
+      if (VEC && !BK) {            // rows of D (sdj = 1): whole quads, aligned
+        if (j < nj) *reinterpret_cast<float4*>(d) = make_float4(r[0], r[1], r[2], r[3]);
+      } else {
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          if (j + y < nj) d[y * sdj] = r[y];
+      }
+    }
+  }
+}
+
 // out[e] = sum_z parts[z][e] (FP64, z in order) - v[e % K]  (B - v 1^T, column-major K x nt)
 template <typename R>
 __global__ void k_coeff_center_parts(const R* __restrict__ parts, int nsplit, const double* __restrict__ v, int K,
@@ -237,6 +408,21 @@ cudaError_t gemm(int ni, int nj, int64_t nk, const R* A, int64_t sai, int64_t sa
   const int64_t kper = ((nk + nsplit - 1) / nsplit + 15) / 16 * 16;
   dim3 grid((unsigned)((ni + 63) / 64), (unsigned)((nj + 63) / 64), (unsigned)nsplit);
   k_gemm_simt<R><<<grid, 256, 0, s>>>(ni, nj, nk, A, sai, sak, B, sbk, sbj, D, sdi, sdj, dsplit, beta, kper);
+  return cudaGetLastError();
+}
+
+// FP32 form of the products (k_gemm_f32): the quads' strides and bases are checked
+// here; `vec` says whether the sizes allow them.
+template <bool BK>
+cudaError_t gemm_f32(int ni, int nj, int64_t nk, const float* A, int64_t sai, const float* B, int64_t ldb, float* D,
+                     int64_t sdi, int64_t sdj, const double* mean, int nsplit, int64_t dsplit, cudaStream_t s) {
+  const int64_t kper = ((nk + nsplit - 1) / nsplit + 15) / 16 * 16;
+  const dim3 grid((unsigned)((nj + 127) / 128), (unsigned)((ni + 63) / 64), (unsigned)nsplit);
+  const uintptr_t bases = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(D);
+  // rows of A (and of B, or of B and D) in whole quads
+  const bool vec = bases % 16 == 0 && sai % 4 == 0 && ldb % 4 == 0 && nk % 4 == 0 && (BK || (nj % 4 == 0 && sdi % 4 == 0));
+  if (vec) k_gemm_f32<BK, true><<<grid, 128, 0, s>>>(ni, nj, nk, A, sai, B, ldb, D, sdi, sdj, dsplit, mean, kper);
+  else k_gemm_f32<BK, false><<<grid, 128, 0, s>>>(ni, nj, nk, A, sai, B, ldb, D, sdi, sdj, dsplit, mean, kper);
   return cudaGetLastError();
 }
 
@@ -277,21 +463,68 @@ struct Scratch {
   }
 };
 
-// P_w, P_b (K x M, type R) of the selected modes.
+// The Gram and its inverse beside the product over the points: they keep the FP64
+// pipe and one SM busy, the product the FP32 pipe, and neither needs the other
+// (K = 64, nt = 4096, M = 65 536: 0.86 + 0.16 ms beside 0.97).  The side stream is the
+// plan's copy stream, joined again whatever happens, before the scratch is given
+// back; a call under stream capture stays on its own stream.
+struct Fork {
+  cudaStream_t s = nullptr, side = nullptr;
+  cudaEvent_t ev = nullptr;
+  bool open = false;
+  // the stream to run beside s on (s itself when there is none to fork to)
+  cudaStream_t begin(spod_plan_s& p, cudaStream_t s_) {
+    s = s_;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return s;
+    }
+    if (!p.h2d_stream && cudaStreamCreateWithFlags(&p.h2d_stream, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaGetLastError();
+      p.h2d_stream = nullptr;
+      return s;
+    }
+    if (p.host_ev.empty()) {
+      if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        return s;
+      }
+      p.host_ev.push_back(ev);
+    }
+    ev = p.host_ev[0];
+    side = p.h2d_stream;
+    if (cudaEventRecord(ev, s) != cudaSuccess || cudaStreamWaitEvent(side, ev, 0) != cudaSuccess) {
+      cudaGetLastError();
+      return s;
+    }
+    open = true;
+    return side;
+  }
+  cudaError_t join() {
+    if (!open) return cudaSuccess;
+    open = false;
+    cudaError_t e = cudaEventRecord(ev, side);
+    return e == cudaSuccess ? cudaStreamWaitEvent(s, ev, 0) : e;
+  }
+  ~Fork() { join(); }
+};
+
+// P_w (unless Pw is NULL) and P_b (K x M, type R) of the selected modes.
 template <typename R>
 cudaError_t build_basis(const spod_plan_s& p, const void* d_Phi, int nmodes, const std::vector<BasisRow>& rows,
                         Scratch& sc, R** Pw, R** Pb, cudaStream_t s) {
   const int K = (int)rows.size();
   const int64_t M = p.M;
   BasisRow* d_rows = static_cast<BasisRow*>(sc.get(sizeof(BasisRow) * K));
-  *Pw = static_cast<R*>(sc.get(sizeof(R) * (size_t)K * M));
+  if (Pw) *Pw = static_cast<R*>(sc.get(sizeof(R) * (size_t)K * M));
   *Pb = static_cast<R*>(sc.get(sizeof(R) * (size_t)K * M));
   if (sc.err != cudaSuccess) return sc.err;
   cudaError_t e = cudaMemcpyAsync(d_rows, rows.data(), sizeof(BasisRow) * K, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)std::min<int64_t>((M + 255) / 256, 1024), (unsigned)K);
   k_coeff_basis<R><<<grid, 256, 0, s>>>(static_cast<const R*>(d_Phi), nmodes, M, d_rows,
-                                        static_cast<const R*>(p.d_sqrtW), *Pw, *Pb);
+                                        static_cast<const R*>(p.d_sqrtW), Pw ? *Pw : nullptr, *Pb);
   return cudaGetLastError();
 }
 
@@ -321,14 +554,26 @@ cudaError_t coeffs_t(spod_plan_s& p, const void* d_X, const void* d_Phi, int nmo
   if (sc.err != cudaSuccess) return sc.err;
   e = cudaMemcpyAsync(d_q, qrows.data(), sizeof(int2) * qrows.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
-  // G and v
-  k_coeff_gram<R><<<dim3((unsigned)K, (unsigned)(K + 1)), 256, 0, s>>>(Pw, Pb, p.d_mu, M, K, G, v);
+  // G and v, and G^{-1}, beside the product
+  Fork fork;
+  cudaStream_t sg = fork.begin(p, s);
+  const unsigned kt = (unsigned)((K + 3) / 4);
+  k_coeff_gram<R><<<dim3(kt, kt + 1), 256, 0, sg>>>(Pw, Pb, p.d_mu, M, K, G, v);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_spd_inverse<<<1, 1024, sizeof(double) * K, s>>>(G, Ginv, K, p.d_flags);
+  const int inv_smem = K <= kInvSmemK;
+  const size_t inv_bytes = sizeof(double) * ((size_t)K + (inv_smem ? 2 * (size_t)K * (K + 1) : 0));
+  e = cudaFuncSetAttribute(k_spd_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_bytes);
+  if (e != cudaSuccess) return e;
+  k_spd_inverse<<<1, 1024, inv_bytes, sg>>>(G, Ginv, K, inv_smem, p.d_flags);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // B = P_w X^T (column-major K x nt; X[t][m]), per split of the points, then B - v 1^T in FP64
-  e = gemm<R>(K, (int)nt, M, Pw, M, 1, static_cast<const R*>(d_X), 1, M, B, 1, K, (R)0, nsplit, (int64_t)K * nt, s);
+  if constexpr (sizeof(R) == 4)
+    e = gemm_f32<true>(K, (int)nt, M, Pw, M, static_cast<const float*>(d_X), M, B, 1, K, nullptr, nsplit,
+                       (int64_t)K * nt, s);
+  else
+    e = gemm<R>(K, (int)nt, M, Pw, M, 1, static_cast<const R*>(d_X), 1, M, B, 1, K, (R)0, nsplit, (int64_t)K * nt, s);
   if (e != cudaSuccess) return e;
+  if ((e = fork.join()) != cudaSuccess) return e;
   k_coeff_center_parts<R><<<1024, 256, 0, s>>>(B, nsplit, v, K, (int64_t)K * nt, B64);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // C = G^{-1} (B - v 1^T)  (FP64, column-major K x nt)
@@ -349,8 +594,8 @@ cudaError_t reconstruct_t(spod_plan_s& p, const void* d_Phi, int nmodes, int nmo
   const int64_t M = p.M, nt = p.nt;
   Scratch sc;
   sc.s = s;
-  R *Pw = nullptr, *Pb = nullptr;
-  cudaError_t e = build_basis<R>(p, d_Phi, nmodes, rows, sc, &Pw, &Pb, s);
+  R* Pb = nullptr;
+  cudaError_t e = build_basis<R>(p, d_Phi, nmodes, rows, sc, nullptr, &Pb, s);
   if (e != cudaSuccess) return e;
   R* C = static_cast<R*>(sc.get(sizeof(R) * (size_t)K * nt));
   int2* d_q = static_cast<int2*>(sc.get(sizeof(int2) * qrows.size()));
@@ -361,10 +606,14 @@ cudaError_t reconstruct_t(spod_plan_s& p, const void* d_Phi, int nmodes, int nmo
   k_coeff_unpack<R><<<pg, 256, 0, s>>>(reinterpret_cast<const double2*>(d_A), d_q, K, nt, C);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   R* X = static_cast<R*>(d_Xrec);
-  k_fill_mean<R><<<2048, 256, 0, s>>>(p.d_mu, M, M * nt, X);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // X[t][m] += sum_r C[t][r] P_b[r][m]  (C column-major K x nt, P_b rows of M)
-  return gemm<R>((int)nt, (int)M, K, C, K, 1, Pb, M, 1, X, M, 1, (R)1, 1, 0, s);
+  // X[t][m] = mu[m] + sum_r C[t][r] P_b[r][m]  (C column-major K x nt, P_b rows of M)
+  if constexpr (sizeof(R) == 4) {
+    return gemm_f32<false>((int)nt, (int)M, K, C, K, Pb, M, X, M, 1, p.d_mu, 1, 0, s);
+  } else {
+    k_fill_mean<R><<<2048, 256, 0, s>>>(p.d_mu, M, M * nt, X);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return gemm<R>((int)nt, (int)M, K, C, K, 1, Pb, M, 1, X, M, 1, (R)1, 1, 0, s);
+  }
 }
 
 }  // namespace

@@ -211,7 +211,14 @@ template <typename R> struct Cplx;
 template <> struct Cplx<float> { using T = float2; };
 template <> struct Cplx<double> { using T = double2; };
 
-template <typename R, int KG>
+//
+// What bounds it (FP32): instruction issue.  The two points of a thread are the two
+// lanes of packed FMAs (fma.rn.f32x2, each lane rounded as a scalar FMA: the same
+// results), with B_f staged as (re, re, im, im) so that a mode costs one 16-byte
+// broadcast load and four packed FMAs where it cost an 8-byte load and eight FMAs:
+// 128 x 128 x 3 points, nb = 38, 257 bins, 38 modes
+// 4.05 -> 3.14 ms.
+template <typename R, int KG, bool kPacked>
 __global__ void __launch_bounds__(128) k_modes_simt(const R* __restrict__ qhat, int64_t rs, int nb, int nmodes,
                                                     int nmp, int64_t mcount, int64_t m0, int64_t M,
                                                     const R* __restrict__ bmat, const R* __restrict__ scale,
@@ -219,13 +226,17 @@ __global__ void __launch_bounds__(128) k_modes_simt(const R* __restrict__ qhat, 
   using V2 = typename Cplx<R>::T;
   const int f = f0 + blockIdx.y;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  static_assert(!kPacked || sizeof(R) == 4, "packed FMAs are FP32");
   V2* sB = reinterpret_cast<V2*>(smem_raw);                       // [nb][nmp]
+  float4* sB4 = reinterpret_cast<float4*>(smem_raw);              // packed: [nb][nmp] (re, re, im, im)
   const V2* Bf = reinterpret_cast<const V2*>(bmat) + (size_t)f * nb * nmodes;
   for (int e = threadIdx.x; e < nb * nmp; e += blockDim.x) {
     const int l = e / nmp, k = e - l * nmp;
     V2 z;
     z.x = 0; z.y = 0;
-    sB[e] = k < nmodes ? Bf[l * nmodes + k] : z;
+    if (k < nmodes) z = Bf[l * nmodes + k];
+    if constexpr (kPacked) sB4[e] = make_float4(z.x, z.x, z.y, z.y);
+    else sB[e] = z;
   }
   __syncthreads();
   const int64_t lm = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2;
@@ -238,24 +249,48 @@ __global__ void __launch_bounds__(128) k_modes_simt(const R* __restrict__ qhat, 
   const bool vec = (M % 2) == 0;                                  // two points = one aligned 2-complex store
   for (int k0 = 0; k0 < nmodes; k0 += KG) {
     R ar0[KG], ai0[KG], ar1[KG], ai1[KG];
+    if constexpr (kPacked) {
+      float2 ar[KG], ai[KG];
 #pragma unroll
-    for (int j = 0; j < KG; ++j) { ar0[j] = 0; ai0[j] = 0; ar1[j] = 0; ai1[j] = 0; }
-    for (int l = 0; l < nb; ++l) {
-      const V2 qr = *reinterpret_cast<const V2*>(qf + (int64_t)l * rs);        // Re, points lm and lm + 1
-      const V2 qi = *reinterpret_cast<const V2*>(qf + (int64_t)(nb + l) * rs); // Im
-      const V2* bl = sB + l * nmp + k0;
+      for (int j = 0; j < KG; ++j) ar[j] = ai[j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+      for (int l = 0; l < nb; ++l) {
+        const float2 qr = *reinterpret_cast<const float2*>(qf + (int64_t)l * rs);
+        const float2 qi = *reinterpret_cast<const float2*>(qf + (int64_t)(nb + l) * rs);
+        const float2 qn = make_float2(-qi.x, -qi.y);
+        const float4* bl = sB4 + l * nmp + k0;
 #pragma unroll
-      for (int j = 0; j < KG; ++j) {
-        const V2 b = bl[j];
-        // q * b as FMA chains (four FMAs per complex product and point)
-        ar0[j] = fma(qr.x, b.x, ar0[j]);
-        ar0[j] = fma(-qi.x, b.y, ar0[j]);
-        ai0[j] = fma(qr.x, b.y, ai0[j]);
-        ai0[j] = fma(qi.x, b.x, ai0[j]);
-        ar1[j] = fma(qr.y, b.x, ar1[j]);
-        ar1[j] = fma(-qi.y, b.y, ar1[j]);
-        ai1[j] = fma(qr.y, b.y, ai1[j]);
-        ai1[j] = fma(qi.y, b.x, ai1[j]);
+        for (int j = 0; j < KG; ++j) {
+          const float4 b = bl[j];
+          const float2 br = make_float2(b.x, b.y), bi = make_float2(b.z, b.w);
+          ar[j] = __ffma2_rn(qr, br, ar[j]);
+          ar[j] = __ffma2_rn(qn, bi, ar[j]);
+          ai[j] = __ffma2_rn(qr, bi, ai[j]);
+          ai[j] = __ffma2_rn(qi, br, ai[j]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < KG; ++j) { ar0[j] = ar[j].x; ar1[j] = ar[j].y; ai0[j] = ai[j].x; ai1[j] = ai[j].y; }
+    } else {
+#pragma unroll
+      for (int j = 0; j < KG; ++j) { ar0[j] = 0; ai0[j] = 0; ar1[j] = 0; ai1[j] = 0; }
+      for (int l = 0; l < nb; ++l) {
+        const V2 qr = *reinterpret_cast<const V2*>(qf + (int64_t)l * rs);        // Re, points lm and lm + 1
+        const V2 qi = *reinterpret_cast<const V2*>(qf + (int64_t)(nb + l) * rs); // Im
+        const V2* bl = sB + l * nmp + k0;
+#pragma unroll
+        for (int j = 0; j < KG; ++j) {
+          const V2 b = bl[j];
+          // q * b as FMA chains (four FMAs per complex product and point)
+          ar0[j] = fma(qr.x, b.x, ar0[j]);
+          ar0[j] = fma(-qi.x, b.y, ar0[j]);
+          ai0[j] = fma(qr.x, b.y, ai0[j]);
+          ai0[j] = fma(qi.x, b.x, ai0[j]);
+          ar1[j] = fma(qr.y, b.x, ar1[j]);
+          ar1[j] = fma(-qi.y, b.y, ar1[j]);
+          ai1[j] = fma(qr.y, b.y, ai1[j]);
+          ai1[j] = fma(qi.y, b.x, ai1[j]);
+        }
       }
     }
 #pragma unroll
@@ -319,45 +354,49 @@ cudaError_t launch_mode_coeffs(const spod_plan_s& p, int nmodes, cudaStream_t s)
 }
 
 #ifndef SPOD_MODES_KGMAX
-#define SPOD_MODES_KGMAX 16
+#define SPOD_MODES_KGMAX 19
 #endif
 // Modes per group of the FP32 kernel: the fewest groups of at most
-// SPOD_MODES_KGMAX modes, split evenly (38 modes: 13 + 13 + 12 instead of
-// 16 + 16 + 6 with six idle slots of the last group's FMAs per point).
-template <typename R, int KG>
-static cudaError_t modes_kernel(void (**kern)(const R*, int64_t, int, int, int, int64_t, int64_t, int64_t, const R*,
-                                              const R*, R*, int, int64_t, int64_t)) {
-  *kern = k_modes_simt<R, KG>;
-  return cudaSuccess;
+// SPOD_MODES_KGMAX modes, split evenly (38 modes: 19 + 19; three groups of 13 read
+// the points' Qhat once more and measured 3.17 ms against 3.14).
+template <typename R>
+using ModesKern = void (*)(const R*, int64_t, int, int, int, int64_t, int64_t, int64_t, const R*, const R*, R*, int,
+                           int64_t, int64_t);
+template <int KG>
+static ModesKern<float> modes_f32(bool packed) {
+  return packed ? k_modes_simt<float, KG, true> : k_modes_simt<float, KG, false>;
 }
 
 template <typename R>
 static cudaError_t launch_modes_t(const spod_plan_s& p, int64_t m0, int64_t mcount, int nmodes, void* d_Phi,
                                   cudaStream_t s, int* nlaunch, bool adjoint, int f0, int f1, int64_t qoff,
                                   int64_t out_ld, int64_t out_off) {
-  void (*kern)(const R*, int64_t, int, int, int, int64_t, int64_t, int64_t, const R*, const R*, R*, int, int64_t,
-               int64_t) = nullptr;
+  ModesKern<R> kern = nullptr;
   int KG = 8;
+  bool packed = false;
   if constexpr (sizeof(R) == 8) {
-    modes_kernel<R, 8>(&kern);
+    kern = k_modes_simt<R, 8, false>;
   } else {
     const int groups = (nmodes + SPOD_MODES_KGMAX - 1) / SPOD_MODES_KGMAX;
     const int need = (nmodes + groups - 1) / groups;
-    constexpr int kChoices[] = {4, 8, 10, 13, 16, 20};
+    constexpr int kChoices[] = {4, 8, 10, 13, 16, 19};
     KG = SPOD_MODES_KGMAX;
     for (int c : kChoices)
       if (c >= need && c <= SPOD_MODES_KGMAX) { KG = c; break; }
+    // packed FMAs while B_f at 16 bytes an entry leaves room for four CTAs per SM
+    // (the 8-byte form for more blocks and modes, up to what fits at all)
+    packed = 16 * (size_t)p.nb * ((nmodes + KG - 1) / KG * KG) <= 56 * 1024;
     switch (KG) {
-      case 4: modes_kernel<R, 4>(&kern); break;
-      case 8: modes_kernel<R, 8>(&kern); break;
-      case 10: modes_kernel<R, 10>(&kern); break;
-      case 13: modes_kernel<R, 13>(&kern); break;
-      case 16: modes_kernel<R, 16>(&kern); break;
-      default: modes_kernel<R, SPOD_MODES_KGMAX>(&kern); KG = SPOD_MODES_KGMAX; break;
+      case 4: kern = modes_f32<4>(packed); break;
+      case 8: kern = modes_f32<8>(packed); break;
+      case 10: kern = modes_f32<10>(packed); break;
+      case 13: kern = modes_f32<13>(packed); break;
+      case 16: kern = modes_f32<16>(packed); break;
+      default: kern = modes_f32<SPOD_MODES_KGMAX>(packed); KG = SPOD_MODES_KGMAX; break;
     }
   }
   const int nmp = (nmodes + KG - 1) / KG * KG;
-  const size_t smem = sizeof(typename Cplx<R>::T) * (size_t)p.nb * nmp;
+  const size_t smem = (packed ? 16 : sizeof(typename Cplx<R>::T)) * (size_t)p.nb * nmp;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   constexpr int threads = 128;

@@ -19,10 +19,15 @@ namespace spod {
 namespace {
 
 constexpr int TK = 32;        // points staged per round
-constexpr int KSUB = 4;       // thread groups splitting a round's points (point k goes to group k % KSUB)
-constexpr int TPG = 64;       // threads per group: one 4x4 complex tile of the upper triangle each
-constexpr int kThreads = KSUB * TPG;
-// FP32 -> FP64 promotion every 64 rounds (TK * 64 / KSUB = 512 points a
+constexpr int kThreads = 256;
+// Threads per group: one 4x4 complex tile of the upper triangle each; kThreads / TPG
+// groups split a round's points (point k goes to group k % KSUB).  FP64 is bound by
+// its pipe, which a warp instruction occupies as long whatever its active lanes:
+// with few tiles (nb = 15: 10) groups of 64 left most lanes idle, so FP64 takes the
+// smallest group of 16, 32 or 64 that holds the tiles (64 x 32 points, 129 bins,
+// nb = 15: 1.00 -> 0.63 ms).  FP32 keeps 64 (its partial sums round with the split).
+constexpr int tpg_of(int ntiles, bool f64) { return !f64 ? 64 : ntiles <= 16 ? 16 : ntiles <= 32 ? 32 : 64; }
+// FP32 -> FP64 promotion every 64 rounds (TK * 64 / 4 = 512 points a
 // thread): FP64 adds issue at a small fraction of the FP32 rate on this part,
 // so the promotion is kept rare; round-to-nearest FP32 runs of 512 products
 // keep the partial sums to ~sqrt(512) 2^-24 relative
@@ -61,11 +66,12 @@ __device__ __forceinline__ void load4(const double* p, double* v) {
 // added into FP64 sums in shared memory every kFlushRounds rounds, and the
 // KSUB groups' FP64 sums are combined in group order at the end (for FP64 the
 // combining area overlays the staging buffers, which are idle by then).
-template <typename R>
+template <typename R, int TPG>
 __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_gram_simt(const R* __restrict__ qhat, int64_t rs, int nb,
                                                            int64_t mcount, int64_t per_split, int first, int nbuf,
                                                            double* __restrict__ gpart, int nf) {
   constexpr bool kPromote = sizeof(R) == 4;
+  constexpr int KSUB = kThreads / TPG;
   const int s = blockIdx.x;
   const int f = blockIdx.y;
   const int ntl = (nb + 3) / 4;
@@ -182,16 +188,36 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_gram_simt(
         load4(sI + k * RS + 4 * I, xi);
         load4(sR + k * RS + 4 * J, yr);
         load4(sI + k * RS + 4 * J, yi);
+        // conj(x_i) * y_j as four FMAs (the sums' rounding order is the FMAs'); FP32
+        // takes two j at a time in packed FMAs, each lane rounded as a scalar one
+        if constexpr (kPromote) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+          for (int i = 0; i < 4; ++i) {
+            const float2 x2 = make_float2(xr[i], xr[i]), z2 = make_float2(xi[i], xi[i]);
+            const float2 n2 = make_float2(-xi[i], -xi[i]);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            // conj(x_i) * y_j as four FMAs (the sums' rounding order is the FMAs')
-            ar[i][j] = fma(xr[i], yr[j], ar[i][j]);
-            ar[i][j] = fma(xi[i], yi[j], ar[i][j]);
-            ai[i][j] = fma(xr[i], yi[j], ai[i][j]);
-            ai[i][j] = fma(-xi[i], yr[j], ai[i][j]);
+            for (int j = 0; j < 4; j += 2) {
+              const float2 yr2 = make_float2(yr[j], yr[j + 1]), yi2 = make_float2(yi[j], yi[j + 1]);
+              float2 tr = make_float2(ar[i][j], ar[i][j + 1]), ti = make_float2(ai[i][j], ai[i][j + 1]);
+              tr = __ffma2_rn(x2, yr2, tr);
+              tr = __ffma2_rn(z2, yi2, tr);
+              ti = __ffma2_rn(x2, yi2, ti);
+              ti = __ffma2_rn(n2, yr2, ti);
+              ar[i][j] = tr.x; ar[i][j + 1] = tr.y;
+              ai[i][j] = ti.x; ai[i][j + 1] = ti.y;
+            }
           }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              ar[i][j] = fma(xr[i], yr[j], ar[i][j]);
+              ar[i][j] = fma(xi[i], yi[j], ar[i][j]);
+              ai[i][j] = fma(xr[i], yi[j], ai[i][j]);
+              ai[i][j] = fma(-xi[i], yr[j], ai[i][j]);
+            }
+        }
       }
       if (kPromote && (r + 1) % kFlushRounds == 0) flush();
     }
@@ -281,10 +307,15 @@ template <typename R>
 cudaError_t launch_gram_t(const spod_plan_s& p, int64_t mcount, bool first, cudaStream_t s) {
   const int ntl = (p.nb + 3) / 4;
   const int ntiles = ntl * (ntl + 1) / 2;
-  const int groups = (ntiles + TPG - 1) / TPG;
+  const int tpg = tpg_of(ntiles, sizeof(R) == 8);
+  const int groups = (ntiles + tpg - 1) / tpg;
   size_t smem = 0;
   const int nbuf = gram_simt_nbuf(p.nb, sizeof(R), &smem);
-  auto kern = k_gram_simt<R>;
+  auto kern = k_gram_simt<R, 64>;
+  if constexpr (sizeof(R) == 8) {
+    if (tpg == 16) kern = k_gram_simt<R, 16>;
+    if (tpg == 32) kern = k_gram_simt<R, 32>;
+  }
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int64_t per = (mcount + p.gram_splits - 1) / p.gram_splits;
