@@ -441,6 +441,246 @@ __global__ void __launch_bounds__(256, 2) k_adjoint512(const float2* __restrict_
   }
 }
 
+// ---------------------------------------------------------------- nfft = 256, 384, 720, FP32
+// The same adjoint in two register passes, N = RA RB, n = k1 + RA k2:
+//   pass A   thread (column, n2), n2 < RB, takes the RA entries RB n1 + n2, an RA-point
+//            DFT, the twiddle W_N^(n2 k1), and stores over them;
+//   pass B   thread (column, k1), k1 < RA, takes its RB values, an RB-point DFT, and
+//            has the time samples n = k1 + RA k2 of its point pair: windowed, each is
+//            the first contribution to its row (stored to the ring), one of the
+//            middle ones (added) or the last (added to the ring's, the mean taken off
+//            and written to dL/dX), so that the rows need no pass of their own.
+// What bounds it: the read of R and the write of dL/dX, with the transform's issue
+// close behind; the Stockham form (k_adjoint) took two shared-memory accesses per
+// element and radix, a cleared ring and a separate pass over the finished rows:
+// 256 x 128 x 2 points, nt = 4096, nfft 256, nb = 31, one spod_backward call (R written by
+// the mode kernel and read here): 3.03 -> 1.78 ms.
+template <int N> struct AdjTwo;
+template <> struct AdjTwo<256> { static constexpr int RA = 16, RB = 16, TP = 32; };
+template <> struct AdjTwo<384> { static constexpr int RA = 24, RB = 16, TP = 32; };
+template <> struct AdjTwo<720> { static constexpr int RA = 24, RB = 30, TP = 16; };
+
+// RAD-point forward DFT in registers.  24 = 3 x 8 and 30 = 2 x 3 x 5 by the prime
+// factor map (Good 1958): with n = 8 a + 3 q mod 24, W_24^(n k) = W_3^(a k) W_8^(q k),
+// so X[k] is entry (k mod 3, k mod 8) of a 3 x 8 transform with no twiddles.
+template <int RAD>
+__device__ __forceinline__ void adj_dft(float2* v) {
+  if constexpr (RAD == 16) {
+    adj_dft16(v);
+  } else if constexpr (RAD == 24) {
+    float2 t[3][8];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) t[a][q] = v[(8 * a + 3 * q) % 24];
+      dft_small<8, float2, float>(t[a]);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      float2 u[3] = {t[0][q], t[1][q], t[2][q]};
+      dft_small<3, float2, float>(u);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v[(16 * a + 9 * q) % 24] = u[a];     // k = a mod 3, q mod 8
+    }
+  } else {
+    static_assert(RAD == 30, "no register DFT of this length");
+    float2 t[2][3][5];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) t[a][b][c] = v[(15 * a + 10 * b + 6 * c) % 30];
+        dft_small<5, float2, float>(t[a][b]);
+      }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        float2 u[3] = {t[a][0][c], t[a][1][c], t[a][2][c]};
+        dft_small<3, float2, float>(u);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) t[a][b][c] = u[b];
+      }
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        v[(10 * b + 6 * c) % 30] = cadd(t[0][b][c], t[1][b][c]);       // k = a mod 2, b mod 3, c mod 5
+        v[(15 + 10 * b + 6 * c) % 30] = csub(t[0][b][c], t[1][b][c]);
+      }
+    }
+  }
+}
+
+template <int N>
+struct AdjGeo {
+  using F = AdjTwo<N>;
+  static constexpr int RA = F::RA, RB = F::RB, TP = F::TP, C = TP / 2;
+  static constexpr int THREADS = RB * C, PB = RB;           // PB: threads per column
+  static constexpr int NF = N / 2 + 1;
+  static constexpr int IT = (NF + PB - 1) / PB;             // bins per thread
+  static constexpr size_t smem = sizeof(float2) * ((size_t)N * C + N) +
+                                 sizeof(float) * ((size_t)N + (size_t)N * TP + TP + (size_t)PB * TP);
+  static_assert(N == RA * RB, "two passes");
+};
+
+template <int N>
+__global__ void __launch_bounds__(AdjGeo<N>::THREADS, 2) k_adjoint_two(const float2* __restrict__ Rsp, int64_t rs,
+                                                                       const float* __restrict__ win,
+                                                                       const float2* __restrict__ tw_g,
+                                                                       const float2* __restrict__ wc_g,
+                                                                       float* __restrict__ dX, AdjArgs a) {
+  using G = AdjGeo<N>;
+  constexpr int RA = G::RA, RB = G::RB, TP = G::TP, C = G::C, PB = G::PB, NF = G::NF, IT = G::IT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* const buf = reinterpret_cast<float2*>(smem_raw);   // [N][C]
+  float2* const tw = buf + (size_t)N * C;                    // [N]
+  float* const wsm = reinterpret_cast<float*>(tw + N);       // [N]
+  float* const ring = wsm + N;                               // [N][TP]
+  float* const mean = ring + (size_t)N * TP;                 // [TP]
+  float* const red = mean + TP;                              // [PB][TP]
+  const int S = a.step, tid = threadIdx.x;
+  const int col = tid % C, b0 = tid / C;
+  const int64_t lm0 = (int64_t)blockIdx.x * TP;
+  const int64_t gm0 = a.m0 + lm0;
+  const int64_t rm0 = gm0 - a.roff;
+  const bool ok0 = lm0 + 2 * col < a.mcount, ok1 = lm0 + 2 * col + 1 < a.mcount;
+  for (int i = tid; i < N; i += G::THREADS) {
+    tw[i] = tw_g[i];
+    wsm[i] = win[i];
+  }
+  // bins b0 + PB it of the thread's point pair: block l of R (rows past the points as zeros)
+  const float2* const rbase = Rsp + rm0 + 2 * col;
+  float4 pr[IT];
+  auto load_block = [&](int l) {
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int f = b0 + PB * it;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (f < NF) {
+        const float2* const p = rbase + ((int64_t)f * a.ncol + l) * rs;
+        if (ok1) v = *reinterpret_cast<const float4*>(p);    // an even column of an aligned row
+        else if (ok0) { const float2 x = p[0]; v.x = x.x; v.y = x.y; }
+      }
+      pr[it] = v;
+    }
+  };
+  load_block(0);
+  // ---- mean of dL/dxt per point: (1/nt) sum_l Re(sum_f R[f][l][m] Wc_f), from R's
+  // extra column when it has one
+  {
+    float m0 = 0.f, m1 = 0.f;
+    if (a.ncol > a.nb) {
+      for (int f = b0; f < NF; f += PB) {
+        const float2* const p = rbase + ((int64_t)f * a.ncol + a.nb) * rs;
+        if (ok0) m0 += p[0].x;
+        if (ok1) m1 += p[1].x;
+      }
+    } else {
+      for (int f = b0; f < NF; f += PB) {
+        const float2 w = wc_g[f];
+        for (int l = 0; l < a.nb; ++l) {
+          const float2* const p = rbase + ((int64_t)f * a.ncol + l) * rs;
+          if (ok0) { m0 = fmaf(p[0].x, w.x, m0); m0 = fmaf(-p[0].y, w.y, m0); }
+          if (ok1) { m1 = fmaf(p[1].x, w.x, m1); m1 = fmaf(-p[1].y, w.y, m1); }
+        }
+      }
+    }
+    red[b0 * TP + 2 * col] = m0;
+    red[b0 * TP + 2 * col + 1] = m1;
+    __syncthreads();
+    if (tid < TP) {
+      float sm = 0.f;
+      for (int k = 0; k < PB; ++k) sm += red[k * TP + tid];
+      mean[tid] = a.subtract_mean ? (float)(sm * a.inv_nt) : 0.f;
+    }
+    __syncthreads();
+  }
+  const float mean0 = mean[2 * col], mean1 = mean[2 * col + 1];
+  float* const dcol = dX + gm0 + 2 * col;
+  const bool pair = ok1 && a.M % 2 == 0;                     // (the points' first one is even)
+  auto write = [&](int64_t t, float v0, float v1) {
+    float* const d = dcol + t * a.M;
+    if (pair) {
+      *reinterpret_cast<float2*>(d) = make_float2(v0, v1);
+    } else {
+      if (ok0) d[0] = v0;
+      if (ok1) d[1] = v1;
+    }
+  };
+  int rb = 0;                                                // ring slot of the block's first row
+  for (int l = 0; l < a.nb; ++l) {
+    // ---- conj of the packed Hermitian extension (as in k_adjoint)
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int f = b0 + PB * it;
+      if (f >= NF) break;
+      const float4 r = pr[it];
+      if (f == 0 || 2 * f == N) {                            // H = R + conj R
+        buf[f * C + col] = make_float2(r.x, -r.z);
+      } else {
+        buf[f * C + col] = make_float2(0.5f * (r.x - r.w), -0.5f * (r.y + r.z));
+        buf[(N - f) * C + col] = make_float2(0.5f * (r.x + r.w), -0.5f * (r.z - r.y));
+      }
+    }
+    if (l + 1 < a.nb) load_block(l + 1);
+    __syncthreads();
+    {                                                        // pass A: n2 = b0
+      float2 v[RA];
+#pragma unroll
+      for (int n1 = 0; n1 < RA; ++n1) v[n1] = buf[(RB * n1 + b0) * C + col];
+      adj_dft<RA>(v);
+#pragma unroll
+      for (int k1 = 1; k1 < RA; ++k1) v[k1] = adj_cmul(v[k1], tw[b0 * k1]);
+#pragma unroll
+      for (int k1 = 0; k1 < RA; ++k1) buf[(RB * k1 + b0) * C + col] = v[k1];
+    }
+    __syncthreads();
+    const int64_t tb = (int64_t)l * S;
+    const bool first = l == 0, last = l + 1 == a.nb;
+#pragma unroll
+    for (int i = 0; i < (RA + PB - 1) / PB; ++i) {           // pass B
+      const int k1 = b0 + PB * i;
+      if (RA % PB != 0 && k1 >= RA) break;
+      float2 v[RB];
+#pragma unroll
+      for (int n2 = 0; n2 < RB; ++n2) v[n2] = buf[(RB * k1 + n2) * C + col];
+      adj_dft<RB>(v);
+#pragma unroll
+      for (int k2 = 0; k2 < RB; ++k2) {
+        const int n = k1 + RA * k2;
+        const float cw = wsm[n];
+        int slot = rb + n;
+        if (slot >= N) slot -= N;
+        float2* const rp = reinterpret_cast<float2*>(ring + slot * TP + 2 * col);
+        float2 acc = make_float2(0.f, 0.f);
+        if (!first && n < N - S) acc = *rp;                  // rows an earlier block holds too
+        acc.x = fmaf(cw, v[k2].x, acc.x);
+        acc.y = fmaf(-cw, v[k2].y, acc.y);
+        if (last || n < S) write(tb + n, acc.x - mean0, acc.y - mean1);   // no later block holds the row
+        else *rp = acc;
+      }
+    }
+    __syncthreads();
+    rb += S;
+    if (rb >= N) rb -= N;
+  }
+  // the uncovered tail (gradient 0 before projection)
+  for (int64_t t = (int64_t)(a.nb - 1) * S + N + b0; t < a.nt; t += PB) write(t, -mean0, -mean1);
+}
+
+template <int N>
+cudaError_t launch_adjoint_two(const spod_plan_s& p, const AdjArgs& a, const void* d_R, int64_t rs, void* d_dX,
+                               cudaStream_t s) {
+  using G = AdjGeo<N>;
+  cudaError_t e = cudaFuncSetAttribute(k_adjoint_two<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem);
+  if (e != cudaSuccess) return e;
+  const int64_t grid = (a.mcount + G::TP - 1) / G::TP;
+  k_adjoint_two<N><<<(unsigned)grid, G::THREADS, G::smem, s>>>(
+      static_cast<const float2*>(d_R), rs, static_cast<const float*>(p.d_win), static_cast<const float2*>(p.d_tw),
+      static_cast<const float2*>(p.d_wc), static_cast<float*>(d_dX), a);
+  return cudaGetLastError();
+}
+
 size_t adjoint512_smem_bytes(int nf) {
   return sizeof(float2) * ((size_t)2 * kAdjN * kAdjC + kAdjN + nf) +
          sizeof(float) * ((size_t)kAdjN * kAdjTP + kAdjTP + 256);
@@ -489,13 +729,18 @@ cudaError_t launch_adj_gmat(const spod_plan_s& p, const double* d_g, cudaStream_
 
 cudaError_t launch_adjoint_chunk(const spod_plan_s& p, const void* d_R, int64_t rs, int64_t roff, int64_t m0,
                                  int64_t mcount, void* d_dX, cudaStream_t s) {
-  if (!p.f64 && p.nfft == kAdjN) {
+  if (!p.f64 && (p.nfft == 256 || p.nfft == 384 || p.nfft == kAdjN || p.nfft == 720)) {
     AdjArgs a;
     a.M = p.M; a.m0 = m0; a.mcount = mcount; a.nt = p.nt; a.roff = roff;
     a.nfft = p.nfft; a.step = p.step; a.nb = p.nb; a.nf = p.nf; a.ncol = p.adj_cols;
     a.subtract_mean = p.desc.subtract_mean;
     a.inv_nt = 1.0 / (double)p.nt;
     a.fp = p.fft;
+    // (the columns of R and dL/dX that a tile starts at are even: m0 and roff are
+    // multiples of 64, the rows of R of 128 points)
+    if (p.nfft == 256) return launch_adjoint_two<256>(p, a, d_R, rs, d_dX, s);
+    if (p.nfft == 384) return launch_adjoint_two<384>(p, a, d_R, rs, d_dX, s);
+    if (p.nfft == 720) return launch_adjoint_two<720>(p, a, d_R, rs, d_dX, s);
     const size_t smem = adjoint512_smem_bytes(p.nf);
     cudaError_t e = cudaFuncSetAttribute(k_adjoint512, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
