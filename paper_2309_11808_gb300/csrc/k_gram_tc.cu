@@ -37,7 +37,7 @@
 // and the warps that sum the lo squares load a block's rows in one batch.  bf16x3,
 // 361 x 720 x 2 points: nb = 7, 361 bins 11.5 -> 4.1 ms (now 55 cycles per N = 16 MMA
 // bound it), nb = 21, 193 bins 6.2 -> 3.0 (5.7 TB/s of Qhat); 512 x 256 x 3 points,
-// nb = 38, 257 bins 6.8 -> 5.0 (6.2 TB/s); BF16, nb = 33, 129 bins 4.2 -> 2.9.
+// nb = 38, 257 bins 6.8 -> 4.8 (6.5 TB/s); BF16, nb = 33, 129 bins 4.2 -> 2.7.
 //
 // Persistent CTAs (one per SM by default) walk a contiguous range of the
 // f-major list of (frequency, block pair) entries, up to KPB / 2 pairs an item.  Warp 8 issues TMA into a
@@ -114,12 +114,45 @@ __device__ __forceinline__ void kahan_add2(float& s0, float& s1, float& c0, floa
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+               "%12, %13, %14, %15}, [%16];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+                 "=f"(v[7]), "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]),
+                 "=f"(v[14]), "=f"(v[15])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+               "%12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, "
+               "%30, %31}, [%32];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+                 "=f"(v[7]), "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]),
+                 "=f"(v[14]), "=f"(v[15]), "=f"(v[16]), "=f"(v[17]), "=f"(v[18]), "=f"(v[19]), "=f"(v[20]),
+                 "=f"(v[21]), "=f"(v[22]), "=f"(v[23]), "=f"(v[24]), "=f"(v[25]), "=f"(v[26]), "=f"(v[27]),
+                 "=f"(v[28]), "=f"(v[29]), "=f"(v[30]), "=f"(v[31])
+               : "r"(taddr));
+}
+// N consecutive columns of this thread's lane (no wait), in the fewest loads: each
+// tcgen05.ld costs about as much whatever its width, and they bound the drains
+// (BF16, nb = 33, 129 bins, 361 x 720 x 2 points: 2.93 ms in loads of 8 columns, 2.71
+// so, 4.84 in loads of 4 by twice the warps).
+template <int N>
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float* v) {
+  if constexpr (N >= 32) {
+    tmem_ld32(taddr, v);
+    if constexpr (N > 32) tmem_ld_cols<N - 32>(taddr + 32u, v + 32);
+  } else if constexpr (N >= 16) {
+    tmem_ld16(taddr, v);
+    if constexpr (N > 16) tmem_ld_cols<N - 16>(taddr + 16u, v + 16);
+  } else {
+    static_assert(N == 8, "columns in eights");
+    tmem_ld8(taddr, v);
+  }
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -437,7 +470,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
     // ---------------- epilogue: TMEM -> registers -> slots.  Warp (quad,
     // half) drains rows quad*32 .. +31 and the HC columns of its half; of A1
     // (symmetric) only the 8-column chunks that reach the upper triangle
-    // (some row of the quad <= some column of the chunk) are read and summed.
+    // (some row of the quad <= some column of the chunk) are summed.
     constexpr int CH = HC / 8;
     const int quad = warp & 3, half = warp >> 2;
     const int row = quad * 32 + lane;
@@ -487,9 +520,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
 #pragma unroll
           for (int r = 0; r < LB; ++r)
             if (r0 + r <= gw.run) {
-#pragma unroll
-              for (int c = 0; c < CH; ++c)
-                if (c >= c_first) tmem_ld8(t1 + (uint32_t)((r0 + r) * NP + c * 8), v[r] + c * 8);
+              tmem_ld_cols<HC>(t1 + (uint32_t)((r0 + r) * NP), v[r]);
             }
           tmem_wait_ld();
           if (r0 + LB > gw.run) {                  // the group's last batch: the buffer is free
@@ -532,8 +563,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
           const uint32_t t2 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((a.nacc * HB + a2b) * NP) +
                               (uint32_t)col0;
           float v[HC];
-#pragma unroll
-          for (int c = 0; c < CH; ++c) tmem_ld8(t2 + (uint32_t)(c * 8), v + c * 8);
+          tmem_ld_cols<HC>(t2, v);
           tmem_wait_ld();
           tc_fence_before();
           mbar_arrive(smem_u32(&hdr->a2empty[a2b]));
