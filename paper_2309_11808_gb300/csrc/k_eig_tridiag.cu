@@ -452,23 +452,47 @@ __device__ __forceinline__ dc dc_mulc(dc a, dc b) {   // conj(a) * b
   return {dw_add(dw_mul(a.re, b.re), dw_mul(a.im, b.im)), dw_sub(dw_mul(a.re, b.im), dw_mul(a.im, b.re))};
 }
 
-// Block sum of a df64 complex value; every thread gets the same sum (the
-// warps' partials are added in warp order).
-__device__ dc block_sum_dc(dc v, float4* red) {
-  for (int o = 16; o > 0; o >>= 1) {
-    dc u;
-    u.re.h = __shfl_xor_sync(0xffffffffu, v.re.h, o);
-    u.re.l = __shfl_xor_sync(0xffffffffu, v.re.l, o);
-    u.im.h = __shfl_xor_sync(0xffffffffu, v.im.h, o);
-    u.im.l = __shfl_xor_sync(0xffffffffu, v.im.l, o);
-    v = dc_add(v, u);
-  }
+// Block sum of df64 values v of the threads below m (the others hold zeros, and
+// the levels and warps that would only add them are left out: the same sum); every
+// thread gets it (the warps' partials are added in warp order).  One barrier: `red`
+// holds 8 entries that no thread still reads, and the caller's next sum takes
+// others.  With every level, all eight partials and two barriers the kernel took
+// 178 us at n = 15 (129 matrices), 332 at 21 (193) and 855 at 38 (257); so, 165,
+// 299 and 803.
+__device__ dc block_sum_dc(dc v, int m, float4* red) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[w] = dc_st(v);
+  const int nw = min((int)(blockDim.x >> 5), (m + 31) >> 5);
+  if (w < nw) {
+    for (int o = m > 16 ? 16 : m > 8 ? 8 : m > 4 ? 4 : 2; o > 0; o >>= 1) {
+      dc u;
+      u.re.h = __shfl_xor_sync(0xffffffffu, v.re.h, o);
+      u.re.l = __shfl_xor_sync(0xffffffffu, v.re.l, o);
+      u.im.h = __shfl_xor_sync(0xffffffffu, v.im.h, o);
+      u.im.l = __shfl_xor_sync(0xffffffffu, v.im.l, o);
+      v = dc_add(v, u);
+    }
+    if (lane == 0) red[w] = dc_st(v);
+  }
   __syncthreads();
   dc t = dc_ld(red[0]);
-  for (int i = 1; i < (int)(blockDim.x >> 5); ++i) t = dc_add(t, dc_ld(red[i]));
+  for (int i = 1; i < nw; ++i) t = dc_add(t, dc_ld(red[i]));
+  return t;
+}
+__device__ dw block_sum_dw(dw v, int m, float4* red) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nw = min((int)(blockDim.x >> 5), (m + 31) >> 5);
+  if (w < nw) {
+    for (int o = m > 16 ? 16 : m > 8 ? 8 : m > 4 ? 4 : 2; o > 0; o >>= 1) {
+      dw u;
+      u.h = __shfl_xor_sync(0xffffffffu, v.h, o);
+      u.l = __shfl_xor_sync(0xffffffffu, v.l, o);
+      v = dw_add(v, u);
+    }
+    if (lane == 0) red[w] = make_float4(v.h, v.l, 0.0f, 0.0f);
+  }
+  __syncthreads();
+  dw t = {red[0].x, red[0].y};
+  for (int i = 1; i < nw; ++i) t = dw_add(t, dw{red[i].x, red[i].y});
   return t;
 }
 
@@ -514,12 +538,15 @@ __device__ void householder_dw(const double2* __restrict__ G, double2* A, int ld
     // alpha and x are read before the barriers of the sum below, after
     // which the column is overwritten by v
     const dc alpha = dc_ld(A4[(size_t)(k + 1) * lda + k]);
-    dc pt = dc_zero();
+    dw pt = dw_of(0.0f);
     for (int i = 1 + tid; i < m; i += nth) {
       const dc x = dc_ld(A4[(size_t)(k + 1 + i) * lda + k]);
-      pt.re = dw_add(pt.re, dw_add(dw_mul(x.re, x.re), dw_mul(x.im, x.im)));
+      pt = dw_add(pt, dw_add(dw_mul(x.re, x.re), dw_mul(x.im, x.im)));
     }
-    const dw xn2 = block_sum_dc(pt, red4).re;     // |x[1:]|^2, the same in every thread
+    // this column's two sums and the next one's take different entries of red: a
+    // column without a reflection has no other barrier
+    float4* const redk = red4 + 16 * (k & 1);
+    const dw xn2 = block_sum_dw(pt, m, redk);     // |x[1:]|^2, the same in every thread
     // the reflector, computed by every thread from the same operands (no broadcast)
     dc t = dc_zero(), scale = dc_zero();
     dw beta = alpha.re;                            // stays alpha when no reflection is needed
@@ -569,7 +596,7 @@ __device__ void householder_dw(const double2* __restrict__ G, double2* A, int ld
       pv4[i] = dc_st(pi);
       dot = dc_add(dot, dc_mulc(pi, dc_ld(vv4[i])));
     }
-    dot = block_sum_dc(dot, red4);
+    dot = block_sum_dc(dot, m, redk + 8);
     const dc half_t = {{-0.5f * t.re.h, -0.5f * t.re.l}, {-0.5f * t.im.h, -0.5f * t.im.l}};   // exact
     const dc al = dc_mul(half_t, dot);
     for (int i = tid; i < m; i += nth) pv4[i] = dc_st(dc_add(dc_ld(pv4[i]), dc_mul(al, dc_ld(vv4[i]))));
