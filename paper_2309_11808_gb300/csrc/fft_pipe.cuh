@@ -107,12 +107,11 @@ struct PipeArgs {
   int step, nb, nf, boxr;
   int subtract_mean;
   int qrows;                         // Qhat rows per frequency (blocked layout)
-  // time mean folded into the transform (real data): a provisional centre
+  // time mean folded into the transform (FOLD, real data): a provisional centre
   // c (the mean of kCentreSamples evenly spaced snapshots of the column) is
   // subtracted instead of the mean, the sum of x - c over all nt snapshots
   // accumulated, mu = c + mean(x - c) written to mu_out and
   // rho = sqrt(W) mean(x - c) to Qhat row 2 nb of every frequency
-  int fold;
   int64_t nt, tail0;                 // snapshots; first snapshot in no block
   const void* xg;                    // X itself (tail samples), row stride xld, column of point lm: xc0 + lm
   int64_t xld, xc0;
@@ -253,7 +252,9 @@ __device__ __forceinline__ void stage_a(const Tin* __restrict__ ring, int rb, in
     else if (slot >= N) slot -= N;
     const float2 x = PairLoad<Tin>::get(ring + slot * G::PTP + 2 * col);
     const float wn = wsm[n];
-    const float d0 = (x.x - mhi0) - mlo0, d1 = (x.y - mhi1) - mlo1;
+    // (the folded mean's centre is one float: known at compile time, 720 takes
+    // 5.09 ms for 5.32, 384 6.71 for 6.94, 256 with BF16 5.10 for 5.29)
+    const float d0 = FOLD ? x.x - mhi0 : (x.x - mhi0) - mlo0, d1 = FOLD ? x.y - mhi1 : (x.y - mhi1) - mlo1;
     if (FOLD && n1 >= n1thr) {           // a snapshot no earlier block held
       acc0 += d0;
       acc1 += d1;
@@ -493,7 +494,7 @@ struct PipeLayout : PipeBytes<Tin, TP, N, CPLX, pipe_nbuf<Tin, TP, N, CPLX>()> {
                                TP <= Stages<N, CPLX>::WMAX;
 };
 
-template <typename Tin, int OUTK, int TP, int N, bool CPLX>
+template <typename Tin, int OUTK, int TP, int N, bool CPLX, bool FOLD>
 __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CPLX>()) k_fft_pipe(const __grid_constant__ CUtensorMap xmap,
                                                           const float* __restrict__ win,
                                                           const float2* __restrict__ tw_g,
@@ -570,8 +571,8 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
   // of a column is the mean of its ncen snapshots at rows crow[k]; partial sum b
   // of a column takes k = b, b + kPart, ...  The loads for tile t + t_step are issued
   // while tile t runs (pc0 / pc1) and reduced at its end.
-  constexpr bool FOLDK = !CPLX && OUTK != OUT_NATIVE;
-  const bool fold = FOLDK && a.fold;
+  static_assert(!FOLD || (!CPLX && OUTK != OUT_NATIVE), "the mean is folded for real data and BF16 output");
+  constexpr bool fold = FOLD;
   constexpr int PB = G::BSTEP;
   const int b0 = tid / PC;
   const Tin* const xg = static_cast<const Tin*>(a.xg);
@@ -615,7 +616,7 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
   float cen0 = 0.f, cen1 = 0.f;      // this thread's column pair: centres of the current tile
   float pc0[NV], pc1[NV];            // partial centre sums of the next tile
   float swr = 0.f, cme = 0.f;        // threads < TP: sqrt(W) and centre of point tid of the tile
-  if (fold) {
+  if constexpr (fold) {
     centre_partial(t_first, pc0, pc1);
     put_centre(pc0, pc1);
     __syncthreads();
@@ -635,10 +636,10 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
                                      // complex data: sqrt(W) of its two points
     {
       const int64_t lm = lm0 + 2 * col;
-      if (a.subtract_mean && !a.fold && lm < a.mcount) {
+      if (a.subtract_mean && !fold && lm < a.mcount) {
         const double d = mu[gm0 + 2 * col]; mhi0 = (float)d; mlo0 = (float)(d - (double)mhi0);
       }
-      if (a.subtract_mean && !a.fold && lm + 1 < a.mcount) {
+      if (a.subtract_mean && !fold && lm + 1 < a.mcount) {
         const double d = mu[gm0 + 2 * col + 1]; mhi1 = (float)d; mlo1 = (float)(d - (double)mhi1);
       }
       const int cp = tid % G::OUTCP;
@@ -652,7 +653,7 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
           sw[q] = (lm0 + 4 * cp + q < a.mcount) ? 0.5f * sqrtW[gm0 + 4 * cp + q] : 0.f;
       }
     }
-    if (fold) {
+    if constexpr (fold) {
       mhi0 = cen0;
       mhi1 = cen1;
       if (tid < PTP) swr = lm0 + tid < a.mcount ? sqrtW[gm0 + tid] : 0.f;
@@ -683,7 +684,7 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
           const int n2 = b0 + i * PB;
           if (RB % PB == 0 || n2 < RB) {
             float2 v[RA];
-            stage_a<Tin, N, TP, CPLX, FOLDK>(ring, rb, n2, v, wsm, tw, mhi0, mlo0, mhi1, mlo1, rthr, s0[i % NV],
+            stage_a<Tin, N, TP, CPLX, FOLD>(ring, rb, n2, v, wsm, tw, mhi0, mlo0, mhi1, mlo1, rthr, s0[i % NV],
                                              s1[i % NV]);
             // one buffer: the previous block's output phase must be done reading
             // it (every thread has a first task: PB <= RB)
@@ -692,7 +693,7 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
             for (int k1 = 0; k1 < RA; ++k1) buf[(k1 * RB + n2) * PC + col] = v[k1];
           }
         }
-        if (fold) {
+        if constexpr (fold) {
 #pragma unroll
           for (int vv = 0; vv < NV; ++vv) {
             if (!in_pass) {
@@ -734,7 +735,7 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
       if (rb >= N) rb -= N;
     }
     if (hdr->abort) break;
-    if (fold) {
+    if constexpr (fold) {
       // the snapshots in no block (the tail): partial sum b of a column takes t = tail0 + b + kPart k
       const int64_t lmA = lm0 + 2 * col;
 #pragma unroll
@@ -807,7 +808,7 @@ constexpr int64_t kBlocksPerLaunch = 1024;
 
 // Complex data (CPLX): m0 and mcount count points; the ring, the mean and the
 // tiles work on the 2M interleaved components.  Adds its launches to *nlaunch.
-template <typename Tin, int OUTK, int TP, int N, bool CPLX>
+template <typename Tin, int OUTK, int TP, int N, bool CPLX, bool FOLD = false>
 cudaError_t launch_pipe_n(const spod_plan_s& p, const CUtensorMap& xmap, const void* d_X, int64_t m0,
                           int64_t mcount, cudaStream_t s, int* nlaunch) {
   constexpr int PTHREADS = Geo<N, TP, CPLX>::THREADS;
@@ -821,7 +822,6 @@ cudaError_t launch_pipe_n(const spod_plan_s& p, const CUtensorMap& xmap, const v
   a.boxr = p.ring_boxr;
   a.subtract_mean = p.desc.subtract_mean;
   a.qrows = p.qrows;
-  a.fold = (!CPLX && p.mean_fold) ? 1 : 0;
   a.nt = p.nt;
   a.tail0 = (int64_t)(p.nb - 1) * p.step + p.nfft;
   a.xg = d_X;
@@ -829,7 +829,7 @@ cudaError_t launch_pipe_n(const spod_plan_s& p, const CUtensorMap& xmap, const v
   a.xc0 = a.m0 - a.xoff;
   a.mu_out = p.d_mu;
   const size_t smem = PipeLayout<Tin, TP, N, CPLX>::dyn;
-  auto kern = k_fft_pipe<Tin, OUTK, TP, N, CPLX>;
+  auto kern = k_fft_pipe<Tin, OUTK, TP, N, CPLX, FOLD>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 1;
@@ -874,17 +874,26 @@ bool pipe_has(int tp) {
   return tp == 32 ? PipeLayout<Tin, 32, N, CPLX>::fits : PipeLayout<Tin, 16, N, CPLX>::fits;
 }
 
+template <typename Tin, int OUTK, int TP, bool CPLX, int N>
+cudaError_t launch_pipe_f(const spod_plan_s& p, const CUtensorMap& xmap, const void* d_X, int64_t m0, int64_t mcount,
+                          cudaStream_t s, int* nlaunch) {
+  if constexpr (!CPLX && OUTK != OUT_NATIVE) {
+    if (p.mean_fold) return launch_pipe_n<Tin, OUTK, TP, N, CPLX, true>(p, xmap, d_X, m0, mcount, s, nlaunch);
+  }
+  return launch_pipe_n<Tin, OUTK, TP, N, CPLX>(p, xmap, d_X, m0, mcount, s, nlaunch);
+}
+
 template <typename Tin, int OUTK, bool CPLX, int N>
 cudaError_t launch_pipe_t(const spod_plan_s& p, const CUtensorMap& xmap, int width, const void* d_X, int64_t m0,
                           int64_t mcount, cudaStream_t s, int* nlaunch) {
   if constexpr (PipeLayout<Tin, 64, N, CPLX>::fits) {
-    if (width == 64) return launch_pipe_n<Tin, OUTK, 64, N, CPLX>(p, xmap, d_X, m0, mcount, s, nlaunch);
+    if (width == 64) return launch_pipe_f<Tin, OUTK, 64, CPLX, N>(p, xmap, d_X, m0, mcount, s, nlaunch);
   }
   if constexpr (PipeLayout<Tin, 32, N, CPLX>::fits) {
-    if (width == 32) return launch_pipe_n<Tin, OUTK, 32, N, CPLX>(p, xmap, d_X, m0, mcount, s, nlaunch);
+    if (width == 32) return launch_pipe_f<Tin, OUTK, 32, CPLX, N>(p, xmap, d_X, m0, mcount, s, nlaunch);
   }
   if (width != 16) return cudaErrorInvalidValue;
-  return launch_pipe_n<Tin, OUTK, 16, N, CPLX>(p, xmap, d_X, m0, mcount, s, nlaunch);
+  return launch_pipe_f<Tin, OUTK, 16, CPLX, N>(p, xmap, d_X, m0, mcount, s, nlaunch);
 }
 
 template <typename Tin, bool CPLX, int N>
