@@ -43,8 +43,8 @@
 // lines.  bf16x3 with the mean inside, against Stockham passes through generic
 // shared-memory pointers (an integer round trip in the alignment of the dynamic
 // array had cost the compiler the address space): 512 x 256 x 3 points, nt = 10 000,
-// nfft 512, 12.6 -> 11.2 ms; 361 x 720 x 2 points, nt = 4380, nfft 384, 10.0 -> 6.9;
-// nt = 2920, nfft 720, 9.8 -> 5.3; BF16 input and output, nfft 256, 8.0 -> 5.3 (6.8 TB/s
+// nfft 512, 12.6 -> 11.2 ms; 361 x 720 x 2 points, nt = 4380, nfft 384, 10.0 -> 6.7;
+// nt = 2920, nfft 720, 9.8 -> 5.1; BF16 input and output, nfft 256, 8.0 -> 5.1 (6.8 TB/s
 // of X and Qhat would take 7.0 / 3.9 / 2.6 / 2.0 ms).
 #pragma once
 
