@@ -353,15 +353,22 @@ cudaError_t launch_mode_coeffs(const spod_plan_s& p, int nmodes, cudaStream_t s)
   return cudaGetLastError();
 }
 
-#ifndef SPOD_MODES_KGMAX
-#define SPOD_MODES_KGMAX 19
-#endif
-// Modes per group of the FP32 kernel: the fewest groups of at most
-// SPOD_MODES_KGMAX modes, split evenly (38 modes: 19 + 19; three groups of 13 read
-// the points' Qhat once more and measured 3.17 ms against 3.14).
+// Modes per group of the FP32 kernel: the fewest groups of at most kgmax modes,
+// split evenly, at the next compiled size.  Packed: 19 (38 modes: 19 + 19; three
+// groups of 13 read the points' Qhat once more and measured 3.17 ms against 3.14).
+// Scalar: 16, whose rows are padded less where shared memory is short.
+constexpr int kKgPacked = 19, kKgScalar = 16;
 template <typename R>
 using ModesKern = void (*)(const R*, int64_t, int, int, int, int64_t, int64_t, int64_t, const R*, const R*, R*, int,
                            int64_t, int64_t);
+static int modes_group(int nmodes, int kgmax) {
+  const int groups = (nmodes + kgmax - 1) / kgmax;
+  const int need = (nmodes + groups - 1) / groups;
+  constexpr int kChoices[] = {4, 8, 10, 13, 16};
+  for (int c : kChoices)
+    if (c >= need) return c;
+  return kgmax;
+}
 template <int KG>
 static ModesKern<float> modes_f32(bool packed) {
   return packed ? k_modes_simt<float, KG, true> : k_modes_simt<float, KG, false>;
@@ -377,22 +384,18 @@ static cudaError_t launch_modes_t(const spod_plan_s& p, int64_t m0, int64_t mcou
   if constexpr (sizeof(R) == 8) {
     kern = k_modes_simt<R, 8, false>;
   } else {
-    const int groups = (nmodes + SPOD_MODES_KGMAX - 1) / SPOD_MODES_KGMAX;
-    const int need = (nmodes + groups - 1) / groups;
-    constexpr int kChoices[] = {4, 8, 10, 13, 16, 19};
-    KG = SPOD_MODES_KGMAX;
-    for (int c : kChoices)
-      if (c >= need && c <= SPOD_MODES_KGMAX) { KG = c; break; }
     // packed FMAs while B_f at 16 bytes an entry leaves room for four CTAs per SM
     // (the 8-byte form for more blocks and modes, up to what fits at all)
+    KG = modes_group(nmodes, kKgPacked);
     packed = 16 * (size_t)p.nb * ((nmodes + KG - 1) / KG * KG) <= 56 * 1024;
+    if (!packed) KG = modes_group(nmodes, kKgScalar);
     switch (KG) {
       case 4: kern = modes_f32<4>(packed); break;
       case 8: kern = modes_f32<8>(packed); break;
       case 10: kern = modes_f32<10>(packed); break;
       case 13: kern = modes_f32<13>(packed); break;
       case 16: kern = modes_f32<16>(packed); break;
-      default: kern = modes_f32<SPOD_MODES_KGMAX>(packed); KG = SPOD_MODES_KGMAX; break;
+      default: kern = k_modes_simt<float, kKgPacked, true>; break;
     }
   }
   const int nmp = (nmodes + KG - 1) / KG * KG;

@@ -21,7 +21,8 @@ def test_coefficient_products(npts, nt, fsel, nr):
     assert np.abs(Xr - Xref).max() <= 1e-4 * np.abs(X).max()
 
 
-@pytest.mark.parametrize("nb,nmodes", [(5, 5), (19, 19), (20, 20), (38, 38), (39, 1), (60, 59), (64, 64)])
+@pytest.mark.parametrize("nb,nmodes", [(5, 5), (19, 19), (20, 20), (38, 38), (39, 1), (60, 59), (64, 64),
+                                       (100, 97), (170, 160)])
 @pytest.mark.parametrize("npts", [257, 770])
 def test_fp32_modes(nb, nmodes, npts):
     # Phi = Qhat B, B from the plan's own eigenpairs: the spectra to a few FP32

@@ -1,5 +1,5 @@
-"""Tensor-core Gram and modes over every row padding: blocks of 16 to 64 rows are
-stacked in one MMA and several tiles share a copy, so ragged point counts and
+"""Tensor-core Gram and modes over every row padding: several blocks of
+few rows share an item of the Gram and several tiles a copy of the modes, so ragged point counts and
 last chunks smaller than the ones before them (whose blocks still hold the
 previous chunk's spectra) are where these kernels can go wrong."""
 import numpy as np
