@@ -612,6 +612,10 @@ __device__ void householder_dw(const double2* __restrict__ G, double2* A, int ld
     }
     __syncthreads();
   }
+  // thread 0 wrote the last column's tau; where that column took no reflection (every
+  // real matrix: DC and Nyquist of real data) no barrier has followed, and thread
+  // n - 2 converts the entry below
+  __syncthreads();
   // the diagonal, then the reflectors (strictly below it) and tau to FP64 in place
   for (int i = tid; i < n; i += nth) {
     const float4 a = A4[(size_t)i * lda + i];
