@@ -698,7 +698,7 @@ cudaError_t launch_adjoint_t(const spod_plan_s& p, const void* d_R, int64_t rs, 
   a.fp = p.fft;
   const size_t smem = adjoint_smem_bytes(p);
   auto kern = k_adjoint<R, TP>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const int64_t grid = (mcount + TP - 1) / TP;
   kern<<<(unsigned)grid, 256, smem, s>>>(static_cast<const typename C2<R>::T*>(d_R), rs,

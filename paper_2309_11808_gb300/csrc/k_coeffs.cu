@@ -562,7 +562,7 @@ cudaError_t coeffs_t(spod_plan_s& p, const void* d_X, const void* d_Phi, int nmo
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int inv_smem = K <= kInvSmemK;
   const size_t inv_bytes = sizeof(double) * ((size_t)K + (inv_smem ? 2 * (size_t)K * (K + 1) : 0));
-  e = cudaFuncSetAttribute(k_spd_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_bytes);
+  e = allow_smem(k_spd_inverse, inv_bytes);
   if (e != cudaSuccess) return e;
   k_spd_inverse<<<1, 1024, inv_bytes, sg>>>(G, Ginv, K, inv_smem, p.d_flags);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -326,7 +326,7 @@ size_t eig_smem_bytes(int nb) {
 
 cudaError_t launch_eig(const spod_plan_s& p, cudaStream_t s) {
   const size_t smem = eig_smem_bytes(p.nb);
-  cudaError_t e = cudaFuncSetAttribute(k_eig_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_eig_jacobi, smem);
   if (e != cudaSuccess) return e;
   k_eig_jacobi<<<p.nf, 256, smem, s>>>(p.d_gram, p.nb, p.d_lam, p.d_psi, p.d_eigws, p.d_flags, 50, 1e-14);
   return cudaGetLastError();
@@ -337,7 +337,7 @@ cudaError_t launch_eig(const spod_plan_s& p, cudaStream_t s) {
 cudaError_t launch_eig_buffers(const double* gram, int nf, int nb, double* lam, double* psi, double* gws,
                                unsigned* flags, cudaStream_t s) {
   const size_t smem = eig_smem_bytes(nb);
-  cudaError_t e = cudaFuncSetAttribute(k_eig_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_eig_jacobi, smem);
   if (e != cudaSuccess) return e;
   k_eig_jacobi<<<nf, 256, smem, s>>>(gram, nb, lam, psi, gws, flags, 50, 1e-14);
   return cudaGetLastError();
@@ -400,7 +400,7 @@ static cudaError_t launch_modes_t(const spod_plan_s& p, int64_t m0, int64_t mcou
   }
   const int nmp = (nmodes + KG - 1) / KG * KG;
   const size_t smem = (packed ? 16 : sizeof(typename Cplx<R>::T)) * (size_t)p.nb * nmp;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   constexpr int threads = 128;
   dim3 grid((unsigned)((mcount + 2 * threads - 1) / (2 * threads)), (unsigned)(f1 - f0));

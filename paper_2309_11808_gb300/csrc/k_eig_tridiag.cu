@@ -843,7 +843,7 @@ size_t eig_tridiag_gws_doubles(int nb, int nf) {
 cudaError_t launch_eig_tridiag(const spod_plan_s& p, cudaStream_t s) {
   const size_t smem = eig_tridiag_smem_bytes(p.nb);
   auto kern = p.f64 ? k_eig_tridiag<false> : k_eig_tridiag<true>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<p.nf, kThreads, smem, s>>>(p.d_gram, p.nb, p.d_lam, p.d_psi, p.d_eigws, p.d_flags,
                                     p.eig_max_iter > 0 ? p.eig_max_iter : kMaxIter);

@@ -205,7 +205,7 @@ cudaError_t launch_fft_t(const spod_plan_s& p, const void* d_X, int64_t m0, int6
   a.fp = p.fft;
   const size_t smem = fft_smem_bytes(p);
   auto kern = k_fft<Tin, R, TP, OUTK, CPLX>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const int64_t ntiles = (a.mpad + PPT - 1) / PPT;
   const int64_t grid = ntiles * p.nb;

@@ -294,7 +294,7 @@ cudaError_t launch_ring_n(const spod_plan_s& p, const CUtensorMap& xmap, int64_t
   a.pst = (int)fft_ring_plane_elems(p);
   const size_t smem = fft_ring_smem_bytes(p);
   auto kern = k_fft_ring<Tin, OUTK, NMAX>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, RTHREADS, smem);

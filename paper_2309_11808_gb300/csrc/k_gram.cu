@@ -316,7 +316,7 @@ cudaError_t launch_gram_t(const spod_plan_s& p, int64_t mcount, bool first, cuda
     if (tpg == 16) kern = k_gram_simt<R, 16>;
     if (tpg == 32) kern = k_gram_simt<R, 32>;
   }
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int64_t per = (mcount + p.gram_splits - 1) / p.gram_splits;
   per = ((per + TK - 1) / TK) * TK;

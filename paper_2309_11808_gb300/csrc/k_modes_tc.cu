@@ -459,13 +459,13 @@ cudaError_t launch_modes_tc_chunk(const spod_plan_s& p, int64_t m0, int64_t mcou
       !make_qhat_map(p, p.d_qlo ? p.d_qlo : p.d_qhat, 2 * a.tiles, nblk, &ml))
     return cudaErrorUnknown;
   if (p.desc.precision == SPOD_PREC_BF16X3) {
-    cudaError_t e = cudaFuncSetAttribute(k_modes_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_modes_tc<true>, smem);
     if (e != cudaSuccess) return e;
     k_modes_tc<true><<<(unsigned)grid, kThreadsModes, smem, s>>>(mh, ml, a,
                                                                  static_cast<const uint8_t*>(p.d_bimg), scale,
                                                                  static_cast<float2*>(d_Phi), p.d_flags);
   } else {
-    cudaError_t e = cudaFuncSetAttribute(k_modes_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_modes_tc<false>, smem);
     if (e != cudaSuccess) return e;
     k_modes_tc<false><<<(unsigned)grid, kThreadsModes, smem, s>>>(mh, mh, a,
                                                                   static_cast<const uint8_t*>(p.d_bimg), scale,

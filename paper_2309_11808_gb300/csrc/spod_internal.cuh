@@ -24,6 +24,20 @@ constexpr int kMaxRadixPasses = 32;
 constexpr int kMaxNb = 1024;           // largest supported block count
 constexpr int kEigSmemMaxNb = 48;      // eigen-solver keeps A and V in shared memory up to here
 
+// Dynamic shared memory of a CTA at most (no kernel that takes this much has static
+// shared memory beside it).
+constexpr size_t kSmemMax = 227 * 1024;
+
+// Allow a kernel whose shared memory depends on the plan's sizes the `bytes` of a
+// launch.  The limit is one per kernel and process: it is always raised to the full
+// kSmemMax, because a limit set to one launch's bytes would refuse the launch of a
+// larger plan that another host thread is about to make.
+template <typename Kern>
+inline cudaError_t allow_smem(Kern kern, size_t bytes) {
+  if (bytes > kSmemMax) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+}
+
 // Qhat layout of one spatial chunk.  FP32/FP64 planes are planar, element
 // (f, row, m) at (f * 2 nb + row) * chunk + m.  The BF16 planes of the
 // tensor-core path are blocked by kQBlock points, [chunk / kQBlock][nf][2 nb]
