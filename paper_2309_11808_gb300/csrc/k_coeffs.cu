@@ -52,13 +52,20 @@ __global__ void k_coeff_basis(const R* __restrict__ phi, int nmodes, int64_t M, 
 // fixed order (thread t takes m = t, t + 256, ..).  What bounds it: the FP64 pipe.  K = 64,
 // M = 65 536: 0.86 ms, against 0.80 with one pair per CTA; but those 4160 CTAs kept the
 // product that runs beside it (Fork) off the SMs, and these 152 leave it most of each.
+// Fewer rows make fewer tiles than SMs, whose CTAs would then walk all the points one
+// FP64 FMA after another while the rest of the chip idles: split z takes the points
+// [z mper, (z + 1) mper) and writes part z of G [gridDim.z][K][K] and v [gridDim.z][K],
+// which k_spd_inverse adds up in order (coeff_gram_splits says how many).
 template <typename R>
 __global__ void __launch_bounds__(256) k_coeff_gram(const R* __restrict__ Pw, const R* __restrict__ Pb,
-                                                    const double* __restrict__ mu, int64_t M, int K,
+                                                    const double* __restrict__ mu, int64_t M, int64_t mper, int K,
                                                     double* __restrict__ G, double* __restrict__ v) {
   __shared__ double red[16][8];
   const int i0 = 4 * blockIdx.x, j0 = 4 * blockIdx.y;
   if (j0 < i0) return;
+  const int64_t m0 = (int64_t)blockIdx.z * mper, m1 = min(M, m0 + mper);
+  G += (int64_t)blockIdx.z * K * K;
+  v += (int64_t)blockIdx.z * K;
   const bool isv = j0 >= K;
   const R *a[4], *b[4];
   for (int q = 0; q < 4; ++q) {                       // rows past K repeat the last one
@@ -71,7 +78,7 @@ __global__ void __launch_bounds__(256) k_coeff_gram(const R* __restrict__ Pw, co
 #pragma unroll
     for (int y = 0; y < 4; ++y) acc[x][y] = 0.0;
   if (!isv) {
-    for (int64_t m = threadIdx.x; m < M; m += 256) {
+    for (int64_t m = m0 + threadIdx.x; m < m1; m += 256) {
       double av[4], bv[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) { av[q] = (double)a[q][m]; bv[q] = (double)b[q][m]; }
@@ -81,7 +88,7 @@ __global__ void __launch_bounds__(256) k_coeff_gram(const R* __restrict__ Pw, co
         for (int y = 0; y < 4; ++y) acc[x][y] = fma(av[x], bv[y], acc[x][y]);
     }
   } else {
-    for (int64_t m = threadIdx.x; m < M; m += 256) {
+    for (int64_t m = m0 + threadIdx.x; m < m1; m += 256) {
       const double c = mu[m];
 #pragma unroll
       for (int x = 0; x < 4; ++x) acc[x][0] = fma((double)a[x][m], c, acc[x][0]);
@@ -112,14 +119,16 @@ __global__ void __launch_bounds__(256) k_coeff_gram(const R* __restrict__ Pw, co
 // Ginv = G^{-1} for the symmetric positive definite G (K x K, FP64) by
 // Gauss-Jordan elimination without pivoting (one CTA; G is overwritten).  A
 // pivot that is not positive (a basis that is not linearly independent)
-// raises FLAG_NOTCONV and leaves Ginv unusable.  At step c the columns of G up to c
+// raises FLAG_NOTCONV and leaves Ginv unusable.  G and v come as nparts parts
+// (k_coeff_gram), added up first; v's total goes to its first part.  At step c the columns of G up to c
 // are those of I already and the columns of Ginv past c still are, so a row is K
 // entries: Ginv's up to c and G's past it.  With smem the two matrices are held in
 // shared memory (K <= kInvSmemK: the elimination is a chain of K short steps, and
 // through L2 each one waited for its loads; K = 64: 0.31 -> 0.16 ms).
 constexpr int kInvSmemK = 96;
-__global__ void __launch_bounds__(1024) k_spd_inverse(double* __restrict__ Gg, double* __restrict__ Ginv_g, int K,
-                                                      int smem, unsigned* __restrict__ flags) {
+__global__ void __launch_bounds__(1024) k_spd_inverse(double* __restrict__ Gg, double* __restrict__ v,
+                                                      double* __restrict__ Ginv_g, int K, int nparts, int smem,
+                                                      unsigned* __restrict__ flags) {
   extern __shared__ double sh[];    // fac [K], then (smem) G and Ginv, rows of K + 1
   double* const fac = sh;
   double* const G = smem ? sh + K : Gg;
@@ -128,9 +137,17 @@ __global__ void __launch_bounds__(1024) k_spd_inverse(double* __restrict__ Gg, d
   const int tid = threadIdx.x, nth = blockDim.x;
   for (int idx = tid; idx < K * K; idx += nth) {
     const int i = idx / K, j = idx - i * K;
-    if (smem) G[i * ld + j] = Gg[idx];
+    double g = Gg[idx];
+    for (int z = 1; z < nparts; ++z) g += Gg[(size_t)z * K * K + idx];
+    G[i * ld + j] = g;
     Ginv[i * ld + j] = i == j ? 1.0 : 0.0;
   }
+  if (nparts > 1)
+    for (int i = tid; i < K; i += nth) {
+      double t = v[i];
+      for (int z = 1; z < nparts; ++z) t += v[(size_t)z * K + i];
+      v[i] = t;
+    }
   __syncthreads();
   for (int c = 0; c < K; ++c) {
     const double piv = G[c * ld + c];
@@ -528,6 +545,15 @@ cudaError_t build_basis(const spod_plan_s& p, const void* d_Phi, int nmodes, con
   return cudaGetLastError();
 }
 
+// Parts of the basis Gram's sums over the points: as many as fill the SMs with the
+// tiles' CTAs, of at least 1024 points each (four a thread).  One from K = 41 on (152
+// SMs), where the tiles alone do.  spod_coeffs, M = 262 144, nt = 300: K = 4 1.77 ms with
+// one part, 0.52 so; K = 16 1.81 and 0.53; K = 32 1.88 and 1.08.
+int coeff_gram_splits(int K, int64_t M, int sms) {
+  const int kt = (K + 3) / 4, tiles = kt * (kt + 1) / 2 + kt;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(sms / tiles, M / 1024));
+}
+
 template <typename R>
 cudaError_t coeffs_t(spod_plan_s& p, const void* d_X, const void* d_Phi, int nmodes, int nmodes_r, int nsel,
                      const int* h_freqs, double* d_A, cudaStream_t s) {
@@ -547,9 +573,10 @@ cudaError_t coeffs_t(spod_plan_s& p, const void* d_X, const void* d_Phi, int nmo
   R* B = static_cast<R*>(sc.get(sizeof(R) * (size_t)K * nt * nsplit));
   double* B64 = static_cast<double*>(sc.get(sizeof(double) * (size_t)K * nt));
   double* C = static_cast<double*>(sc.get(sizeof(double) * (size_t)K * nt));
-  double* G = static_cast<double*>(sc.get(sizeof(double) * (size_t)K * K));
+  const int nz = coeff_gram_splits(K, M, p.num_sms);
+  double* G = static_cast<double*>(sc.get(sizeof(double) * (size_t)nz * K * K));
   double* Ginv = static_cast<double*>(sc.get(sizeof(double) * (size_t)K * K));
-  double* v = static_cast<double*>(sc.get(sizeof(double) * K));
+  double* v = static_cast<double*>(sc.get(sizeof(double) * (size_t)nz * K));
   int2* d_q = static_cast<int2*>(sc.get(sizeof(int2) * qrows.size()));
   if (sc.err != cudaSuccess) return sc.err;
   e = cudaMemcpyAsync(d_q, qrows.data(), sizeof(int2) * qrows.size(), cudaMemcpyHostToDevice, s);
@@ -558,13 +585,13 @@ cudaError_t coeffs_t(spod_plan_s& p, const void* d_X, const void* d_Phi, int nmo
   Fork fork;
   cudaStream_t sg = fork.begin(p, s);
   const unsigned kt = (unsigned)((K + 3) / 4);
-  k_coeff_gram<R><<<dim3(kt, kt + 1), 256, 0, sg>>>(Pw, Pb, p.d_mu, M, K, G, v);
+  k_coeff_gram<R><<<dim3(kt, kt + 1, (unsigned)nz), 256, 0, sg>>>(Pw, Pb, p.d_mu, M, (M + nz - 1) / nz, K, G, v);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int inv_smem = K <= kInvSmemK;
   const size_t inv_bytes = sizeof(double) * ((size_t)K + (inv_smem ? 2 * (size_t)K * (K + 1) : 0));
   e = allow_smem(k_spd_inverse, inv_bytes);
   if (e != cudaSuccess) return e;
-  k_spd_inverse<<<1, 1024, inv_bytes, sg>>>(G, Ginv, K, inv_smem, p.d_flags);
+  k_spd_inverse<<<1, 1024, inv_bytes, sg>>>(G, v, Ginv, K, nz, inv_smem, p.d_flags);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // B = P_w X^T (column-major K x nt; X[t][m]), per split of the points, then B - v 1^T in FP64
   if constexpr (sizeof(R) == 4)
