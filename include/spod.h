@@ -359,12 +359,12 @@ typedef struct {
                              plans) leaves its first pipeline stage unfilled, so the waits on it run
                              out after wait_timeout_us and the fit reports SPOD_ETIMEOUT; 0 (default):
                              off.  No other effect. */
-  int fft_tile_points;    /* pipelined FFT (compiled nfft): spatial points per CTA tile, 16, or 32 for
-                             the widest form the plan has (32 points; 64 where it measured faster),
-                             narrowed for grids with fewer such tiles than SMs; the plan picks 32
-                             where it fits in shared memory.  0 on read: the plan does not use the
-                             pipelined FFT; 0 on write: leave as is.  Changes only the launch shape,
-                             not the results. */
+  int fft_tile_points;    /* pipelined FFT (compiled nfft): spatial points per CTA tile, 16, or 32 (64
+                             where that measured faster and every SM has such a tile).  The plan picks
+                             32 where that form fits in shared memory and every SM has a tile of it,
+                             else 16; a width that was written is kept on every grid.  0 on read: the
+                             plan does not use the pipelined FFT; 0 on write: leave as is.  Changes only
+                             the launch shape, not the results. */
 } spod_tuning;
 
 /* The plan's launch shape into *tuning (host).  No counterpart in the paper. */

@@ -853,17 +853,18 @@ cudaError_t launch_pipe_n(const spod_plan_s& p, const CUtensorMap& xmap, const v
 // Width of the tiles a launch takes (the box width of its X map): up to the
 // plan's choice -- 16 points, or 32 and the widest form there is -- the widest for
 // which every SM has a tile (2048 points, nfft 256: 0.037 ms with 16-point tiles,
-// 0.042 with 32).  WMAX: at nfft 384 one CTA of 64 points takes 6.9 ms where two of 32
-// take 8.5 (361 x 720 x 2 points), at nfft 256 two CTAs of 32 points 5.3 and one of
-// 64 5.7 (their ring and buffers leave room for two buffers, so one CTA's barriers
-// overlap the other's passes).
+// 0.042 with 32); a choice that was set is not narrowed below 32.  WMAX: at nfft 384
+// one CTA of 64 points takes 6.9 ms where two of 32 take 8.5 (361 x 720 x 2 points), at
+// nfft 256 two CTAs of 32 points 5.3 and one of 64 5.7 (their ring and buffers leave
+// room for two buffers, so one CTA's barriers overlap the other's passes).
 template <typename Tin, int N, bool CPLX>
-int pipe_width_n(int choice, int64_t points, int sms) {
+int pipe_width_n(const spod_plan_s& p, int64_t points, int sms) {
+  if (p.pipe_tp < 32) return 16;
   if constexpr (PipeLayout<Tin, 64, N, CPLX>::fits) {
-    if (choice >= 32 && points >= (int64_t)64 * sms) return 64;
+    if (points >= (int64_t)64 * sms) return 64;
   }
   if constexpr (PipeLayout<Tin, 32, N, CPLX>::fits) {
-    if (choice >= 32 && points >= (int64_t)32 * sms) return 32;
+    if (p.pipe_tp_set || points >= (int64_t)32 * sms) return 32;
   }
   return 16;
 }
@@ -923,11 +924,11 @@ PipeLen pipe_len() {
     const int64_t pts = p.cplx ? 2 * points : points;       // components
     const int sms = p.num_sms > 0 ? p.num_sms : 148;
     switch (p.desc.in_dtype) {
-      case SPOD_F64: return pipe_width_n<double, N, false>(p.pipe_tp, pts, sms);
-      case SPOD_F32: return pipe_width_n<float, N, false>(p.pipe_tp, pts, sms);
-      case SPOD_C64: return pipe_width_n<float, N, true>(p.pipe_tp, pts, sms);
-      case SPOD_C128: return pipe_width_n<double, N, true>(p.pipe_tp, pts, sms);
-      default: return pipe_width_n<__nv_bfloat16, N, false>(p.pipe_tp, pts, sms);
+      case SPOD_F64: return pipe_width_n<double, N, false>(p, pts, sms);
+      case SPOD_F32: return pipe_width_n<float, N, false>(p, pts, sms);
+      case SPOD_C64: return pipe_width_n<float, N, true>(p, pts, sms);
+      case SPOD_C128: return pipe_width_n<double, N, true>(p, pts, sms);
+      default: return pipe_width_n<__nv_bfloat16, N, false>(p, pts, sms);
     }
   };
   e.launch = [](const spod_plan_s& p, const CUtensorMap& xmap, int width, const void* d_X, int64_t m0, int64_t mcount,

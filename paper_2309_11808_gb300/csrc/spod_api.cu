@@ -396,6 +396,7 @@ spod_status spod_plan_create(const spod_plan_desc* d, spod_plan_t* out) {
   chunk = std::min<int64_t>(chunk, M);
   chunk = ((chunk + tile - 1) / tile) * tile;
   p->chunk_points = chunk;
+  if (p->pipe_ok) p->pipe_tp = std::min(32, fft_pipe_width(*p, std::min<int64_t>(chunk, M)));
   p->Mpad = ((M + tile - 1) / tile) * tile;
   {
     const int64_t ctas = ((p->cplx ? 2 * M : M) + 255) / 256;
@@ -1246,7 +1247,10 @@ spod_status spod_plan_set_tuning(spod_plan_t p, const spod_tuning* t) {
   p->modes_ctas = t->modes_ctas;
   p->eig_max_iter = t->eig_max_iter;
   p->wait_selftest = t->wait_selftest;
-  if (t->fft_tile_points) p->pipe_tp = t->fft_tile_points;
+  if (t->fft_tile_points) {
+    p->pipe_tp = t->fft_tile_points;
+    p->pipe_tp_set = true;
+  }
   ++p->version;
   return SPOD_OK;
 }
@@ -1411,6 +1415,7 @@ spod_status spod_plan_autotune(spod_plan_t p, const void* d_X, void* stream, spo
       if (fft_pipe_has(*p, tp)) tiles.push_back(tp);
   }
   const int keep_splits = p->gram_splits, keep_tp = p->pipe_tp;
+  const bool keep_set = p->pipe_tp_set;
   const int prof = p->prof;
   p->prof = 0;
   cudaEvent_t e0, e1;
@@ -1434,6 +1439,7 @@ spod_status spod_plan_autotune(spod_plan_t p, const void* d_X, void* stream, spo
   for (int tp : tiles) {
     if (st != SPOD_OK) break;
     p->pipe_tp = tp;
+    p->pipe_tp_set = true;
     ++p->version;
     float ms = 0.f;
     st = time_fit(ms);
@@ -1452,7 +1458,10 @@ spod_status spod_plan_autotune(spod_plan_t p, const void* d_X, void* stream, spo
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   p->gram_splits = st == SPOD_OK ? best_c : keep_splits;
-  if (st != SPOD_OK) p->pipe_tp = keep_tp;
+  if (st != SPOD_OK) {
+    p->pipe_tp = keep_tp;
+    p->pipe_tp_set = keep_set;
+  }
   p->prof = prof;
   ++p->version;
   if (st != SPOD_OK) return st;

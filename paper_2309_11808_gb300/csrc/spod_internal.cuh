@@ -109,6 +109,7 @@ struct spod_plan_s {
   bool mean_fold = false;
   int qrows = 0;              // Qhat rows per frequency: 2 nb (+ 1 with mean_fold)
   int pipe_tp = 16;           // its tile choice: 16 points, or 32 and wider (fft_pipe_width)
+  bool pipe_tp_set = false;   // the choice is the caller's (or the autotuner's): not narrowed
   void* encode_fn = nullptr;  // cuTensorMapEncodeTiled
   int num_sms = 0;
 
