@@ -154,7 +154,6 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float* v) {
     tmem_ld8(taddr, v);
   }
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 struct GramHdr {
   uint64_t full[kMaxStages], empty[kMaxStages], accfull[kMaxAcc], accempty[kMaxAcc], a2empty[2], drain;
@@ -530,6 +529,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
 #pragma unroll
           for (int r = 0; r < LB; ++r)
             if (r0 + r <= gw.run) {
+              tmem_loaded<HC>(v[r]);
 #pragma unroll
               for (int c = 0; c < CH; ++c)
                 if (c >= c_first) {
@@ -565,6 +565,7 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
           float v[HC];
           tmem_ld_cols<HC>(t2, v);
           tmem_wait_ld();
+          tmem_loaded<HC>(v);
           tc_fence_before();
           mbar_arrive(smem_u32(&hdr->a2empty[a2b]));
           float* d2 = reinterpret_cast<float*>(slot + (size_t)a.r2 * a.r2 * 8) + (size_t)row * a.r2 + col0;

@@ -91,7 +91,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // B image of frequency f: rows n < nn (2k: real part of mode k, 2k+1: imaginary
 // part), K index kk < np (l: Re Qhat row l, nb + l: Im Qhat row l), BF16 hi
@@ -358,6 +357,7 @@ __global__ void __launch_bounds__(kThreadsModes, 1) k_modes_tc(const __grid_cons
 #pragma unroll
           for (int c = 0; c < 4; ++c)
             if (c0 + c * 8 < 2 * nm) {                 // four modes
+              tmem_loaded<8>(v + c * 8);
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
                 if (inrange && c0 / 2 + c * 4 + j < nm) *out = make_float2(v[8 * c + 2 * j] * rw, v[8 * c + 2 * j + 1] * rw);
