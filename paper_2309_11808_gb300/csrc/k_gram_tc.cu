@@ -651,8 +651,8 @@ __global__ void k_gram_tc_finish(const double* __restrict__ acc, int nb, int r2,
     }
     return v;
   };
-  const int e = blockIdx.y * blockDim.x + threadIdx.x;   // one entry per thread
-  if (e < nb * nb) {
+  const int n2 = nb * nb, stride = (int)(gridDim.y * blockDim.x);
+  for (int e = (int)(blockIdx.y * blockDim.x + threadIdx.x); e < n2; e += stride) {
     const int i = e / nb, j = e - i * nb;
     const int l = min(i, j), lp = max(i, j);
     double vr = dc(l, lp) + dc(nb + l, nb + lp);
@@ -759,10 +759,19 @@ cudaError_t launch_gram_tc_chunk(const spod_plan_s& p, int64_t mcount, bool firs
   return cudaGetLastError();
 }
 
+// CTAs per frequency.  With the folded mean an entry is a chain of FP64 products: one
+// entry per thread (nb = 41, 257 bins: 27.5 us against 30.6 by one CTA).  Without it the
+// kernel only reads, half of it by columns, which one CTA of a frequency finds in L1:
+// one, or as many as fill the SMs (nb = 64, 257 bins: 56 us by one entry per thread,
+// 21 so; 33 bins 12.3 and 8.2).
+int finish_splits(const spod_plan_s& p) {
+  const int most = (p.nb * p.nb + 255) / 256;
+  return p.mean_fold ? most : std::max(1, std::min(most, p.num_sms / p.nf));
+}
+
 cudaError_t launch_gram_tc_finish(const spod_plan_s& p, cudaStream_t s) {
-  k_gram_tc_finish<<<dim3((unsigned)p.nf, (unsigned)((p.nb * p.nb + 255) / 256)), 256, 0, s>>>(
-      p.d_gacc, p.nb, p.qrows, p.mean_fold ? p.d_what : nullptr, p.kappa,
-                                        p.d_gram, p.d_flags);
+  k_gram_tc_finish<<<dim3((unsigned)p.nf, (unsigned)finish_splits(p)), 256, 0, s>>>(
+      p.d_gacc, p.nb, p.qrows, p.mean_fold ? p.d_what : nullptr, p.kappa, p.d_gram, p.d_flags);
   return cudaGetLastError();
 }
 
