@@ -60,7 +60,7 @@ namespace {
 using namespace fft;
 
 // Stages of the compiled lengths: the radices of stage A (A1, A2), B (B1, B2) and
-// C (C1, C2), 1: none.  N = RA RB, RB = RBB RC.  TPT: threads per point; WMAX:
+// C (C1, C2), 1: none.  N = RA RB, RB = RBB RC.  TPT: threads per point (pipe_tpt); WMAX:
 // points of the widest tile.
 template <int N, bool CPLX> struct Stages;
 template <bool CPLX> struct Stages<256, CPLX> {
@@ -81,8 +81,17 @@ template <bool CPLX> struct Stages<720, CPLX> {
   static constexpr int A1 = 8, A2 = 2, B1 = 3, B2 = 3, C1 = 5, C2 = 1, TPT = 16, WMAX = 32;
 };
 
-// Tile geometry: TP points.
-template <int N, int TP, bool CPLX>
+// Threads per point of a form: the length's, but 16 in tiles of 16 points (small grids:
+// one tile an SM, so the threads are all the latency hiding there is) and for 8-byte
+// input at nfft 384 (whose 32-point ring leaves room for one CTA).  With 8 and 16 threads
+// (nb = 10): F32, 2048 points, nfft 256, bf16x3 28.1 and 24.9 us, F64 41.7 and 32.9; F64,
+// 16 384 points, nfft 384, FP32 221 and 193, bf16x3 275 and 230.
+template <typename Tin, int N, int TP, bool CPLX> constexpr int pipe_tpt() {
+  return TP == 16 || (sizeof(Tin) == 8 && N == 384) ? 16 : Stages<N, CPLX>::TPT;
+}
+
+// Tile geometry: TP points, TPT threads each.
+template <int N, int TP, bool CPLX, int TPT>
 struct Geo {
   using F = Stages<N, CPLX>;
   static constexpr int RA = F::A1 * F::A2, RB = N / RA, RBB = F::B1 * F::B2, RC = RB / RBB;
@@ -90,7 +99,7 @@ struct Geo {
   static_assert(RC == F::C1 * F::C2, "the stages' radices multiply to N");
   static constexpr int PTP = TP;                   // points per tile
   static constexpr int PC = TP / 2;                // complex columns (point pairs)
-  static constexpr int THREADS = F::TPT * TP;
+  static constexpr int THREADS = TPT * TP;
   static constexpr int BSTEP = THREADS / PC;       // threads per column
   static constexpr int NA = (RB + BSTEP - 1) / BSTEP;   // stage-A tasks per thread
   static constexpr int OUTCP = PC / 2;             // column pairs per tile
@@ -239,7 +248,7 @@ template <typename Tin, int N, int TP, bool CPLX, bool FOLD>
 __device__ __forceinline__ void stage_a(const Tin* __restrict__ ring, int rb, int n2, float2* v,
                                         const float* __restrict__ wsm, const float2* __restrict__ tw, float mhi0,
                                         float mlo0, float mhi1, float mlo1, int n1thr, float& acc0, float& acc1) {
-  using G = Geo<N, TP, CPLX>;
+  using G = Geo<N, TP, CPLX, pipe_tpt<Tin, N, TP, CPLX>()>;
   using F = Stages<N, CPLX>;
   constexpr int RA = G::RA, RB = G::RB;
   const int col = threadIdx.x % G::PC;
@@ -274,9 +283,9 @@ __device__ __forceinline__ void stage_a(const Tin* __restrict__ ring, int rb, in
 }
 
 // Stage B, in place: task j = (k, g'').
-template <int N, int TP, bool CPLX>
+template <int N, int TP, bool CPLX, int TPT>
 __device__ __forceinline__ void stage_b(float2* __restrict__ buf, const float2* __restrict__ tw) {
-  using G = Geo<N, TP, CPLX>;
+  using G = Geo<N, TP, CPLX, TPT>;
   using F = Stages<N, CPLX>;
   constexpr int RA = G::RA, RBB = G::RBB, RC = G::RC, PC = G::PC, STEP = G::BSTEP;
   const int col = threadIdx.x % PC;
@@ -363,10 +372,10 @@ __device__ __forceinline__ void store_bin2c(const float4 z, const float (&sw)[4]
 
 // Stage C of one k for the two columns of a pair: X[k + NSC q], q < RC, of column
 // 2 cp (u) and 2 cp + 1 (w).
-template <int N, int TP, bool CPLX>
+template <int N, int TP, bool CPLX, int TPT>
 __device__ __forceinline__ void stage_c(const float4* __restrict__ U4, int k, const float2* __restrict__ tw, float2* u,
                                         float2* w) {
-  using G = Geo<N, TP, CPLX>;
+  using G = Geo<N, TP, CPLX, TPT>;
   using F = Stages<N, CPLX>;
   const float4* const p = U4 + ((k % G::RA) * G::RB + (k / G::RA) * G::RC) * G::OUTCP;
 #pragma unroll
@@ -385,11 +394,11 @@ __device__ __forceinline__ float4 pair4(float2 a, float2 b) { return make_float4
 // Complex data: item k < NSC, the bins k + NSC q.  Real data: item j < NSC / 2,
 // k = j and its mirror NSC - j (X[N - k - NSC q] is entry RC - 1 - q of the mirror);
 // item 0 takes k = 0 and k = NSC / 2, each its own mirror.
-template <int OUTK, int TP, int N, bool CPLX>
+template <int OUTK, int TP, int N, bool CPLX, int TPT>
 __device__ __forceinline__ void output_phase(const float2* __restrict__ U, const float2* __restrict__ tw,
                                              const PipeArgs& a, int l, int64_t lm0, const float (&sw)[4],
                                              void* __restrict__ qout, void* __restrict__ qlo) {
-  using G = Geo<N, TP, CPLX>;
+  using G = Geo<N, TP, CPLX, TPT>;
   constexpr int kCp = G::OUTCP, kStep = G::OUTFSTEP, RC = G::RC, NSC = G::NSC;
   const int cp = threadIdx.x % kCp;
   const float4* const U4 = reinterpret_cast<const float4*>(U) + cp;
@@ -424,14 +433,14 @@ __device__ __forceinline__ void output_phase(const float2* __restrict__ U, const
   } else {
     for (int j = threadIdx.x / kCp; j < kItems; j += kStep) {
       float2 u[RC], w[RC];
-      stage_c<N, TP, CPLX>(U4, j, tw, u, w);
+      stage_c<N, TP, CPLX, TPT>(U4, j, tw, u, w);
       if constexpr (CPLX) {
 #pragma unroll
         for (int q = 0; q < RC; ++q) store_bin2c<OUTK>(pair4(u[q], w[q]), sw, a, o0 + (j + q * NSC) * fstep, qout, qlo);
       } else {
         const int jm = j ? NSC - j : NSC / 2;
         float2 um[RC], wm[RC];
-        stage_c<N, TP, CPLX>(U4, jm, tw, um, wm);
+        stage_c<N, TP, CPLX, TPT>(U4, jm, tw, um, wm);
         if (j) {
 #pragma unroll
           for (int q = 0; q < (RC + 1) / 2; ++q)
@@ -480,12 +489,12 @@ struct PipeBytes {
   static constexpr size_t dyn = end + 1024;                    // alignment slack
 };
 // CTAs per SM aimed at: 512 threads at 128 registers
-template <int TP, int N, bool CPLX> constexpr int pipe_ctas() {
-  return Geo<N, TP, CPLX>::THREADS <= 256 ? 2 : 1;
+template <typename Tin, int TP, int N, bool CPLX> constexpr int pipe_ctas() {
+  return pipe_tpt<Tin, N, TP, CPLX>() * TP <= 256 ? 2 : 1;
 }
 // two transform buffers where they fit beside that many CTAs, else one
 template <typename Tin, int TP, int N, bool CPLX> constexpr int pipe_nbuf() {
-  return PipeBytes<Tin, TP, N, CPLX, 2>::dyn + 1024 <= kPipeSmemMax / pipe_ctas<TP, N, CPLX>() ? 2 : 1;
+  return PipeBytes<Tin, TP, N, CPLX, 2>::dyn + 1024 <= kPipeSmemMax / pipe_ctas<Tin, TP, N, CPLX>() ? 2 : 1;
 }
 template <typename Tin, int TP, int N, bool CPLX>
 struct PipeLayout : PipeBytes<Tin, TP, N, CPLX, pipe_nbuf<Tin, TP, N, CPLX>()> {
@@ -495,7 +504,7 @@ struct PipeLayout : PipeBytes<Tin, TP, N, CPLX, pipe_nbuf<Tin, TP, N, CPLX>()> {
 };
 
 template <typename Tin, int OUTK, int TP, int N, bool CPLX, bool FOLD>
-__global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CPLX>()) k_fft_pipe(const __grid_constant__ CUtensorMap xmap,
+__global__ void __launch_bounds__(pipe_tpt<Tin, N, TP, CPLX>() * TP, pipe_ctas<Tin, TP, N, CPLX>()) k_fft_pipe(const __grid_constant__ CUtensorMap xmap,
                                                           const float* __restrict__ win,
                                                           const float2* __restrict__ tw_g,
                                                           const float* __restrict__ sqrtW,
@@ -504,7 +513,8 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
                                                           unsigned* __restrict__ gflags) {
   using namespace tc;
   using L = PipeLayout<Tin, TP, N, CPLX>;
-  using G = Geo<N, TP, CPLX>;
+  constexpr int TPT = pipe_tpt<Tin, N, TP, CPLX>();
+  using G = Geo<N, TP, CPLX, TPT>;
   constexpr int PTP = G::PTP, PC = G::PC, PTHREADS = G::THREADS;
   extern __shared__ unsigned char smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
@@ -725,11 +735,11 @@ __global__ void __launch_bounds__(Geo<N, TP, CPLX>::THREADS, pipe_ctas<TP, N, CP
           if (a.nb > 1) prefetch(t + t_step, N, a.step);
         }
       }
-      stage_b<N, TP, CPLX>(buf, tw);
+      stage_b<N, TP, CPLX, TPT>(buf, tw);
       __syncthreads();
       // two buffers: the next block's stage A writes the other one, which nobody
       // reads since the barrier after its own block's stage A
-      output_phase<OUTK, TP, N, CPLX>(buf, tw, a, l, lm0, sw, qout, qlo);
+      output_phase<OUTK, TP, N, CPLX, TPT>(buf, tw, a, l, lm0, sw, qout, qlo);
       par ^= 1;
       rb += a.step;
       if (rb >= N) rb -= N;
@@ -811,7 +821,7 @@ constexpr int64_t kBlocksPerLaunch = 1024;
 template <typename Tin, int OUTK, int TP, int N, bool CPLX, bool FOLD = false>
 cudaError_t launch_pipe_n(const spod_plan_s& p, const CUtensorMap& xmap, const void* d_X, int64_t m0,
                           int64_t mcount, cudaStream_t s, int* nlaunch) {
-  constexpr int PTHREADS = Geo<N, TP, CPLX>::THREADS;
+  constexpr int PTHREADS = pipe_tpt<Tin, N, TP, CPLX>() * TP;
   constexpr int64_t K = CPLX ? 2 : 1;          // components per point
   PipeArgs a;
   a.m0 = K * m0; a.mcount = K * mcount; a.chunk = p.chunk_points;
