@@ -361,8 +361,8 @@ typedef struct {
                              off.  No other effect. */
   int fft_tile_points;    /* pipelined FFT (compiled nfft): spatial points per CTA tile, 16, or 32 (64
                              where that measured faster and every SM has such a tile).  The plan picks
-                             32 where that form fits in shared memory and every SM has a tile of it,
-                             else 16; a width that was written is kept on every grid.  0 on read: the
+                             32 where that form fits in shared memory and the grid has the tiles for
+                             it (one per SM; complex FP32 data about half), else 16; a width that was written is kept on every grid.  0 on read: the
                              plan does not use the pipelined FFT; 0 on write: leave as is.  Changes only
                              the launch shape, not the results. */
 } spod_tuning;

@@ -863,7 +863,10 @@ cudaError_t launch_pipe_n(const spod_plan_s& p, const CUtensorMap& xmap, const v
 // Width of the tiles a launch takes (the box width of its X map): up to the
 // plan's choice -- 16 points, or 32 and the widest form there is -- the widest for
 // which every SM has a tile (2048 points, nfft 256: 0.037 ms with 16-point tiles,
-// 0.042 with 32); a choice that was set is not narrowed below 32.  WMAX: at nfft 384
+// 0.042 with 32); a choice that was set is not narrowed below 32.  C64 data takes 32
+// components as soon as 16 would give some SM a second tile (nb = 10, 1300 points, bf16x3:
+// nfft 256 31.2 us with 16, 24.9 with 32, nfft 512 57.6 and 42.8; 1200 points 20.8 and
+// 24.8, 35.8 and 42.9).  WMAX: at nfft 384
 // one CTA of 64 points takes 6.9 ms where two of 32 take 8.5 (361 x 720 x 2 points), at
 // nfft 256 two CTAs of 32 points 5.3 and one of 64 5.7 (their ring and buffers leave
 // room for two buffers, so one CTA's barriers overlap the other's passes).
@@ -874,7 +877,8 @@ int pipe_width_n(const spod_plan_s& p, int64_t points, int sms) {
     if (points >= (int64_t)64 * sms) return 64;
   }
   if constexpr (PipeLayout<Tin, 32, N, CPLX>::fits) {
-    if (p.pipe_tp_set || points >= (int64_t)32 * sms) return 32;
+    const int64_t from = CPLX && sizeof(Tin) == 4 ? (int64_t)16 * sms + 1 : (int64_t)32 * sms;
+    if (p.pipe_tp_set || points >= from) return 32;
   }
   return 16;
 }
