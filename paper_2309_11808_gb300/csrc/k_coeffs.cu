@@ -581,9 +581,21 @@ cudaError_t coeffs_t(spod_plan_s& p, const void* d_X, const void* d_Phi, int nmo
   if (sc.err != cudaSuccess) return sc.err;
   e = cudaMemcpyAsync(d_q, qrows.data(), sizeof(int2) * qrows.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
-  // G and v, and G^{-1}, beside the product
+  // B = P_w X^T (column-major K x nt; X[t][m]), per split of the points, then B - v 1^T in FP64
+  auto product = [&]() {
+    if constexpr (sizeof(R) == 4)
+      return gemm_f32<true>(K, (int)nt, M, Pw, M, static_cast<const float*>(d_X), M, B, 1, K, nullptr, nsplit,
+                            (int64_t)K * nt, s);
+    else
+      return gemm<R>(K, (int)nt, M, Pw, M, 1, static_cast<const R*>(d_X), 1, M, B, 1, K, (R)0, nsplit,
+                     (int64_t)K * nt, s);
+  };
+  // G and v, and G^{-1}, beside the product.  In FP64 the product goes first: both take
+  // the FP64 pipe, and the Gram's CTAs, placed before it, leave the product's unevenly
+  // spread (K = 16, nt = 768, M = 16 384: 2.46 ms, 2.26 so; K = 64, nt = 256: 2.00 and 1.69).
   Fork fork;
   cudaStream_t sg = fork.begin(p, s);
+  if (sizeof(R) == 8 && (e = product()) != cudaSuccess) return e;
   const unsigned kt = (unsigned)((K + 3) / 4);
   k_coeff_gram<R><<<dim3(kt, kt + 1, (unsigned)nz), 256, 0, sg>>>(Pw, Pb, p.d_mu, M, (M + nz - 1) / nz, K, G, v);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -593,13 +605,7 @@ cudaError_t coeffs_t(spod_plan_s& p, const void* d_X, const void* d_Phi, int nmo
   if (e != cudaSuccess) return e;
   k_spd_inverse<<<1, 1024, inv_bytes, sg>>>(G, v, Ginv, K, nz, inv_smem, p.d_flags);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // B = P_w X^T (column-major K x nt; X[t][m]), per split of the points, then B - v 1^T in FP64
-  if constexpr (sizeof(R) == 4)
-    e = gemm_f32<true>(K, (int)nt, M, Pw, M, static_cast<const float*>(d_X), M, B, 1, K, nullptr, nsplit,
-                       (int64_t)K * nt, s);
-  else
-    e = gemm<R>(K, (int)nt, M, Pw, M, 1, static_cast<const R*>(d_X), 1, M, B, 1, K, (R)0, nsplit, (int64_t)K * nt, s);
-  if (e != cudaSuccess) return e;
+  if (sizeof(R) == 4 && (e = product()) != cudaSuccess) return e;
   if ((e = fork.join()) != cudaSuccess) return e;
   k_coeff_center_parts<R><<<1024, 256, 0, s>>>(B, nsplit, v, K, (int64_t)K * nt, B64);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
