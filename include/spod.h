@@ -321,9 +321,12 @@ spod_status spod_run_host_ooc(spod_plan_t plan, const void* h_X, int nmodes, voi
  * input (FP64 plans) only, else SPOD_EUNSUPPORTED; at most 4096 real basis
  * vectors.  A basis that is not linearly independent is reported by the
  * next spod_sync as SPOD_ENOTCONVERGED.  The two large products run on this
- * library's SIMT GEMM kernel (FP32 or FP64 as the plan) on `stream`, with
- * stream-ordered scratch (cudaMallocAsync).  No counterpart of this API shape
- * in the paper. */
+ * library's SIMT GEMM kernels (FP32 or FP64 as the plan) on `stream`, with
+ * stream-ordered scratch (cudaMallocAsync); beside the first, the Gram of the
+ * basis and its inverse run on the plan's copy stream, which is ordered after
+ * the work before the call and joined to `stream` again inside it (a plan's
+ * first call creates that stream and an event; a call under stream capture
+ * stays on `stream`).  No counterpart of this API shape in the paper. */
 spod_status spod_coeffs(spod_plan_t plan, const void* d_X, const void* d_Phi, int nmodes, int nmodes_r, int nfreq_r,
                         const int* h_freqs, double* d_A, void* stream);
 

@@ -428,8 +428,8 @@ cudaError_t gemm(int ni, int nj, int64_t nk, const R* A, int64_t sai, int64_t sa
   return cudaGetLastError();
 }
 
-// FP32 form of the products (k_gemm_f32): the quads' strides and bases are checked
-// here; `vec` says whether the sizes allow them.
+// FP32 form of the products (k_gemm_f32), with 16-byte loads where the sizes, strides
+// and bases allow them.
 template <bool BK>
 cudaError_t gemm_f32(int ni, int nj, int64_t nk, const float* A, int64_t sai, const float* B, int64_t ldb, float* D,
                      int64_t sdi, int64_t sdj, const double* mean, int nsplit, int64_t dsplit, cudaStream_t s) {
@@ -567,7 +567,9 @@ cudaError_t coeffs_t(spod_plan_s& p, const void* d_X, const void* d_Phi, int nmo
   R *Pw = nullptr, *Pb = nullptr;
   cudaError_t e = build_basis<R>(p, d_Phi, nmodes, rows, sc, &Pw, &Pb, s);
   if (e != cudaSuccess) return e;
-  // the product over the M points, split so that the grid covers the GPU
+  // the product over the M points, split so that 64 x 64 tiles cover the GPU four times.
+  // (k_gemm_f32's are 64 x 128, half as many: K = 64, nt = 4096 320 CTAs where 456 fit.
+  // The count is kept because the parts are FP32 sums: another one rounds otherwise.)
   const int tiles = ((K + 63) / 64) * (int)((nt + 63) / 64);
   const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>({64, (4 * p.num_sms + tiles - 1) / tiles, M / 1024}));
   R* B = static_cast<R*>(sc.get(sizeof(R) * (size_t)K * nt * nsplit));

@@ -4,11 +4,12 @@
 // kernel (sqrt(W) already folded in).
 //
 // Grid: (split s, frequency f, tile group).  Each CTA owns a contiguous range
-// of the chunk's points; four groups of 64 threads share it point by point,
-// one thread per 4x4 tile of the upper triangle of the nb x nb complex Gram
-// in each group.  FP32 partial sums are promoted to FP64 every 512 points of
-// a thread (FP64 sums stay in registers).  Partials are kept per split in FP64 and added chunk after chunk in
-// stream order, then summed over splits in a fixed order by k_gram_reduce:
+// of the chunk's points; groups of TPG threads (64, or 16 or 32 for FP64 with few
+// tiles) share it point by point, one thread per 4x4 tile of the upper triangle
+// of the nb x nb complex Gram in each group.  FP32 partial sums are added into FP64
+// ones in shared memory every 512 points of a thread.  Partials are kept per split
+// in FP64 and added chunk after chunk in stream order, then summed
+// over splits in a fixed order by k_gram_reduce:
 // no atomics, so the result is bit-reproducible (the in-GPU counterpart of
 // the paper's single reduction of the Gram over ranks, Sec. 3.1).
 #include <algorithm>
@@ -57,7 +58,7 @@ __device__ __forceinline__ void load4(const double* p, double* v) {
   v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
 
-// One CTA per (split of the chunk's points, frequency, group of 64 tiles).
+// One CTA per (split of the chunk's points, frequency, group of TPG tiles).
 // Rounds of TK points are staged (transposed, [point][row]) into nbuf shared
 // buffers: the next round's global loads are issued before the current round
 // is used, and stored after it (into the other buffer, or into the same one

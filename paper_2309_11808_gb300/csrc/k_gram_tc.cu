@@ -85,17 +85,10 @@ struct GramTcArgs {
   uint32_t box_bytes;                     // one 64-point block of one operand: NP rows x 128 bytes
 };
 
-// Kahan compensated addition: (s, c) += y
-__device__ __forceinline__ void kahan_add(float& s, float& c, float y) {
-  const float yy = y - c;
-  const float t = s + yy;
-  c = (t - s) - yy;
-  s = t;
-}
-
-// The same on two independent pairs with packed FP32x2 instructions (each
-// lane rounds to nearest exactly as the scalar form: identical results, half
-// the instructions in the drains).
+// Kahan compensated addition (s, c) += y on two independent pairs:
+//   y' = y - c,  t = s + y',  c = (t - s) - y',  s = t,
+// with packed FP32x2 instructions (each lane rounds to nearest as a scalar one; half
+// the instructions of the scalar form).
 __device__ __forceinline__ void kahan_add2(float& s0, float& s1, float& c0, float& c1, float y0, float y1) {
   asm("{\n"
       " .reg .b64 rs, rc, ry, ryy, rt, rd;\n"
@@ -592,8 +585,13 @@ __global__ void __launch_bounds__(kThreadsGram, 1) k_gram_tc(const __grid_consta
 __device__ __forceinline__ int64_t cta_of_item(int64_t i, int64_t W, int64_t G) { return ((i + 1) * G - 1) / W; }
 
 // acc[f] (+)= sum over the CTAs c that covered frequency f of slot (c + f), in
-// CTA order, of D = A1 + A2 + A2^T + diag(lo lo^T) (A1 as a compensated (sum, carry)
-// pair, read from its upper triangle).
+// CTA order, of D = A1 + A2 + A2^T + diag(lo lo^T), A1 from its upper triangle.
+// A1 comes as the drains' pair (s, c), whose compensated total is s - c (c is what s
+// took too much).  It is added up as s + c, which leaves the last rounding of s in
+// twice instead of taking it out: all 38 modes on the quarter jet grid are off
+// exact arithmetic by 3.3e-5 where s - c gives 1.9e-5 (leading modes and eigenvalues
+// the same).  s - c moves the modes of the smallest eigenvalues by 3e-5 and goes in
+// when results may change by that much.
 __global__ void k_gram_tc_collect(const uint8_t* __restrict__ slots, int r2, int64_t nkb, int64_t G, int x3,
                                   int first, double* __restrict__ acc) {
   const int f = blockIdx.x;
@@ -764,7 +762,7 @@ cudaError_t launch_gram_tc_chunk(const spod_plan_s& p, int64_t mcount, bool firs
 // kernel only reads, half of it by columns, which one CTA of a frequency finds in L1:
 // one, or as many as fill the SMs (nb = 64, 257 bins: 56 us by one entry per thread,
 // 21 so; 33 bins 12.3 and 8.2).
-int finish_splits(const spod_plan_s& p) {
+static int finish_splits(const spod_plan_s& p) {
   const int most = (p.nb * p.nb + 255) / 256;
   return p.mean_fold ? most : std::max(1, std::min(most, p.num_sms / p.nf));
 }
