@@ -3,7 +3,6 @@ the kernels they share take shared memory by the plan's sizes, and one thread's 
 must not change what the other's may take."""
 import threading
 
-import numpy as np
 import pytest
 import torch
 
